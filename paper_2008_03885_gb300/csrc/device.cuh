@@ -74,11 +74,11 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 // s + c * x in the chosen rounding mode.
 // Value as stored on a level: FP32 levels of the bfloat16 storage trial round it.
 template <typename T>
-__device__ __forceinline__ T rnd(const LevelDev<T>& L, T v) {
+__device__ __forceinline__ T rnd(const LevelGeo<T>& L, T v) {
   return v;
 }
 template <>
-__device__ __forceinline__ float rnd<float>(const LevelDev<float>& L, float v) {
+__device__ __forceinline__ float rnd<float>(const LevelGeo<float>& L, float v) {
   return L.bf16 ? __bfloat162float(__float2bfloat16_rn(v)) : v;
 }
 
@@ -130,13 +130,13 @@ struct RowSum {
 __device__ __forceinline__ bool gbit(const uint32_t* m, int k) { return (m[k >> 5] >> (k & 31)) & 1u; }
 
 template <typename T>
-__device__ __forceinline__ int64_t sidx(const LevelDev<T>& L, int i, int j) {
+__device__ __forceinline__ int64_t sidx(const LevelGeo<T>& L, int i, int j) {
   return (int64_t)j * L.pitch + (L.kind == kRot ? (i >> 1) : i);
 }
 
 // Lattice coordinates of the thread's storage element; false if outside storage.
 template <typename T>
-__device__ __forceinline__ bool thread_node(const LevelDev<T>& L, int& i, int& j) {
+__device__ __forceinline__ bool thread_node(const LevelGeo<T>& L, int& i, int& j) {
   const int q = blockIdx.x * kBX + threadIdx.x;
   j = blockIdx.y * blockDim.y + threadIdx.y;
   if (j >= L.rows || q >= L.cols) return false;
@@ -145,18 +145,18 @@ __device__ __forceinline__ bool thread_node(const LevelDev<T>& L, int& i, int& j
 }
 
 template <typename T>
-__device__ __forceinline__ bool interior(const LevelDev<T>& L, int i, int j) {
+__device__ __forceinline__ bool interior(const LevelGeo<T>& L, int i, int j) {
   return i >= L.lo && i < L.n && j >= L.lo && j < L.n;
 }
 
 template <typename T>
-__device__ __forceinline__ bool is_red(const LevelDev<T>& L, int i, int j) {
+__device__ __forceinline__ bool is_red(const LevelGeo<T>& L, int i, int j) {
   return L.kind == kRot ? (i & 1) : ((i + j) & 1);
 }
 
 // Class index of a node that is not a fast node.
 template <typename T>
-__device__ __forceinline__ int class_of(const LevelDev<T>& L, int i, int j) {
+__device__ __forceinline__ int class_of(const LevelGeo<T>& L, int i, int j) {
   if (L.small) return j * L.clsw + i;
   const int e = L.n - L.per;  // last lattice index a fast stencil may reach
   const int cx = i < L.rx ? i : (i > e - L.rx ? 2 * L.rx - (e - i) : L.rx);
@@ -165,13 +165,13 @@ __device__ __forceinline__ int class_of(const LevelDev<T>& L, int i, int j) {
 }
 
 template <typename T>
-__device__ __forceinline__ bool fast_node(const LevelDev<T>& L, int i, int j) {
+__device__ __forceinline__ bool fast_node(const LevelGeo<T>& L, int i, int j) {
   return i >= L.rx && i <= L.fxe && j >= L.ry && j <= L.fye;
 }
 
 // omega / a_pp of node (i, j).
 template <typename T>
-__device__ __forceinline__ T node_wd(const LevelDev<T>& L, int i, int j) {
+__device__ __forceinline__ T node_wd(const LevelGeo<T>& L, int i, int j) {
   return fast_node(L, i, j) ? L.wd : L.cls_wd[class_of(L, i, j)];
 }
 
@@ -265,7 +265,7 @@ __device__ __forceinline__ T relax_fast(const T (&c)[NT], const int (&dl)[NT], T
 // fast_node with the boundary kind fixed at compile time (the NT kernels run at the
 // register limit; constant bounds keep the Dirichlet instantiation free of spills).
 template <bool PER, typename T>
-__device__ __forceinline__ bool fast_node_c(const LevelDev<T>& L, int i, int j) {
+__device__ __forceinline__ bool fast_node_c(const LevelGeo<T>& L, int i, int j) {
   const int e = L.n - (PER ? 1 : 0);
   return i >= L.rx && i <= e - L.rx && j >= L.ry && j <= e - L.ry;
 }

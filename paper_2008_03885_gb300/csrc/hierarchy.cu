@@ -488,10 +488,12 @@ LevelDev<T> to_dev(const HostLevel& L) {
   d.small = L.small;
   d.clsw = L.clsw;
   d.per = L.per;
+  d.bdata = L.boundary_data;
   d.lo = 1 - L.per;
   d.fxe = L.shape.n - L.per - L.rx;
   d.fye = L.shape.n - L.per - L.ry;
   d.wd = (T)L.wd_fast;
+  for (const int2& e : L.cls) d.maxcnt = std::max(d.maxcnt, (int32_t)e.y);
   for (int k = 0; k < d.nt; ++k) {
     d.c[k] = (T)L.c[k];
     const int dx = L.dxs[k], dy = L.dys[k];
@@ -528,7 +530,7 @@ struct Hier {
   int4* d_prog = nullptr;  // program for a sub-cycle with zero initial guess
   int nops = 0;
   int tail_ctas = 1;       // CTAs in the tail's thread-block cluster
-  int tail_smem = 0;       // > 0: the tail's levels live in shared memory (elements)
+  size_t tail_smem = 0;    // > 0: the tail's levels live in shared memory (bytes)
   std::vector<TileLevel> tiles;  // FP32 levels: TMA tile kernels (tiles.h) where eligible
 };
 
@@ -1074,8 +1076,7 @@ mg_status cycle_level(const Ctx& c, int l, T* U, const T* F, bool zero_init, boo
     const int nops = zero_init ? H.nops : H.nops - 1;
     Bracket b(h, l, MG_KERNEL_SMOOTH, c.s);
     if (H.tail_smem > 0)
-      LAUNCH(h, 1, launch_tail_smem<T>(H.d_tail, H.tail_smem, (int)h->host.size() - H.tail_level, prog, nops,
-                                       c.exact, c.s));
+      LAUNCH(h, 1, launch_tail_smem<T>(H.d_tail, H.tail_smem, prog, nops, c.exact, c.s));
     else LAUNCH(h, 1, launch_tail<T>(H.tail_ctas, H.d_tail, prog, nops, c.exact, c.s));
     return MG_OK;
   }
@@ -1133,7 +1134,7 @@ mg_status cycle_level(const Ctx& c, int l, T* U, const T* F, bool zero_init, boo
   }
   if (l + 1 == lmax) {
     if (H.dense.m > 0)
-      LAUNCH(h, 1, launch_coarsest_dense<T>(H.dense, H.L[lmax], c.exact, H.f[lmax], H.d[lmax], H.u[lmax], c.s));
+      LAUNCH(h, 1, launch_coarsest_dense<T>(H.dense, H.L[lmax], c.exact, H.f[lmax], H.u[lmax], c.s));
     else
       LAUNCH(h, 1, launch_coarsest<T>(H.coarsest_idx, H.coarsest_a, H.coarsest_zero, H.f[lmax], H.u[lmax], c.s));
   } else {
@@ -1301,10 +1302,15 @@ mg_status build_tail(mg_handle* h, int64_t max_unknowns, int64_t smem_elems = 0)
       td.sm_d[l] = off + 3 * e;
       off += 4 * e;
     }
-    if (tail_smem_bytes<T>(off, nl - lt) > kTailSmemMaxBytes) return MG_OK;  // no tail
+    int maxcnt = 1;
+    for (int l = lt; l < nl; ++l) maxcnt = std::max(maxcnt, (int)H.L[l].h.maxcnt);
+    const TailSmemPlan plan = tail_smem_plan<T>(off, maxcnt, H.dense.m);
+    if (plan.octs == 0) return MG_OK;  // no tail
     td.sm_top = lt;
     td.sm_elems = off;
-    H.tail_smem = off;
+    td.sm_octs = plan.octs;
+    td.sm_K = plan.K;
+    H.tail_smem = plan.bytes;
   }
   for (int l = 0; l < nl; ++l) {
     td.L[l] = H.L[l].d;

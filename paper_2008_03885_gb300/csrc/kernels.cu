@@ -15,34 +15,58 @@
 
 #include "kernels.h"
 #include "device.cuh"
+#include "rows.cuh"
 
 namespace nsmg {
 namespace {
 
+// Arguments shared by the half-sweep and residual kernels. The grid is one-dimensional:
+// `sblocks` blocks of octets for the nodes off the fast rectangle (rows.cuh; first, since
+// theirs is the longest chain of loads), then the fast nodes' blocks, gx to a block row.
+template <typename T>
+struct SweepArgs {
+  LevelGeo<T> L;
+  const LevelDev<T>* Lp;
+  StripGeo S;
+  int32_t colour, sblocks, gx, K;
+};
+
+// Terms a lane of an octet fetches at once: rows of the 5/9-point levels have at most 9
+// terms, the wide Galerkin rows up to 45 (longer ones take several batches).
+constexpr int kStripBatchNt = 2, kStripBatchGen = 6;
+
 template <typename T, bool EXACT, int NT, bool PER>
-__global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_half_sweep_nt(const LevelDev<T>* __restrict__ Lp, const T* __restrict__ uin,
-                                const T* __restrict__ f, T* __restrict__ uout, int red) {
+__global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value)
+    k_half_sweep_nt(const __grid_constant__ SweepArgs<T> A, const T* __restrict__ uin, const T* __restrict__ f,
+                    T* __restrict__ uout) {
+  extern __shared__ __align__(16) unsigned char strip_smem[];
   constexpr int kRows = RowsPer<T>::value;
-  const LevelDev<T>& L = *Lp;
+  const LevelGeo<T>& L = A.L;
+  const int red = A.colour;
+  if ((int)blockIdx.x < A.sblocks) {
+    strip_rows<T, EXACT, kStripBatchNt, kRowRelax>(L, A.S, red, blockIdx.x, uin, f, uout, strip_smem, A.K);
+    return;
+  }
+  const int by = ((int)blockIdx.x - A.sblocks) / A.gx, bx = (int)blockIdx.x - A.sblocks - by * A.gx;
   T c[NT];
   int d0[NT], d1[NT];
 #pragma unroll
   for (int k = 0; k < NT; ++k) {
-    c[k] = L.c[k];
-    d0[k] = L.delta[0][k];
-    d1[k] = L.delta[1][k];
+    c[k] = A.Lp->c[k];
+    d0[k] = A.Lp->delta[0][k];
+    d1[k] = A.Lp->delta[1][k];
   }
   const T wd = L.wd;
   const int n = L.n;
   constexpr int lo = PER ? 0 : 1;
-  const int jb = blockIdx.y * (kBY * kRows) + threadIdx.y;
+  const int jb = by * (kBY * kRows) + threadIdx.y;
   // Prefetch the thread's u and f lines of all its rows into L2 before the first row's
   // loads. Measured on GB300 at 4097^2: FP32 axis half-sweep 59.5 -> 55.3 us (order 4),
   // 52.3 -> 45.8 us (order 2); FP64 rotated 178 -> 173 us; no gain (or a loss) for the
   // other two combinations, which skip it.
   if ((sizeof(T) == 4) == (L.kind == kAxis)) {
-    const int col = L.kind == kAxis ? min(2 * (int)(blockIdx.x * kBX + threadIdx.x), n)
-                                    : min((int)(blockIdx.x * kBX + threadIdx.x), L.cols - 1);
+    const int col = L.kind == kAxis ? min(2 * (int)(bx * kBX + threadIdx.x), n)
+                                    : min((int)(bx * kBX + threadIdx.x), L.cols - 1);
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
       const int64_t at = (int64_t)min(jb + r * kBY, L.rows - 1) * L.pitch + col;
@@ -50,8 +74,9 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_half_sweep_n
       prefetch_l2(f + at);
     }
   }
+  const bool fast = !A.S.all;
   if (L.kind == kAxis) {
-    const int i0 = 2 * (blockIdx.x * kBX + threadIdx.x);
+    const int i0 = 2 * (bx * kBX + threadIdx.x);
     if (i0 > n) return;
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
@@ -61,13 +86,12 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_half_sweep_n
       const int ic = 2 * i0 + 1 - i;
       const int64_t row = (int64_t)j * L.pitch;
       if (ic >= lo && ic < n) uout[row + ic] = uin[row + ic];
-      if (i < lo || i >= n) continue;
+      if (!fast || !fast_node_c<PER>(L, i, j)) continue;  // off the fast rectangle: the octets' node
       const int64_t at = row + i;
-      uout[at] = rnd(L, fast_node_c<PER>(L, i, j) ? relax_fast<T, EXACT, NT>(c, d0, wd, uin, f, at)
-                                                  : relax_value<T, EXACT, 1>(L, uin, f, i, j, at));
+      uout[at] = rnd(L, relax_fast<T, EXACT, NT>(c, d0, wd, uin, f, at));
     }
   } else {
-    const int q = blockIdx.x * kBX + threadIdx.x;
+    const int q = bx * kBX + threadIdx.x;
     if (q >= L.cols) return;
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
@@ -80,30 +104,35 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_half_sweep_n
         uout[at] = uin[at];
         continue;
       }
-      uout[at] = rnd(L, fast_node_c<PER>(L, i, j) ? relax_fast<T, EXACT, NT>(c, (i & 1) ? d1 : d0, wd, uin, f, at)
-                                                  : relax_value<T, EXACT, 1>(L, uin, f, i, j, at));
+      if (!fast || !fast_node_c<PER>(L, i, j)) continue;
+      uout[at] = rnd(L, relax_fast<T, EXACT, NT>(c, (i & 1) ? d1 : d0, wd, uin, f, at));
     }
   }
 }
 
 template <typename T, bool EXACT, int NT, bool PER>
-__global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_residual_nt(const LevelDev<T>* __restrict__ Lp, const T* __restrict__ u,
-                              const T* __restrict__ f, T* __restrict__ d) {
+__global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value)
+    k_residual_nt(const __grid_constant__ SweepArgs<T> A, const T* __restrict__ u, const T* __restrict__ f,
+                  T* __restrict__ d) {
+  extern __shared__ __align__(16) unsigned char strip_smem[];
   constexpr int kRows = RowsPer<T>::value;
-  const LevelDev<T>& L = *Lp;
+  const LevelGeo<T>& L = A.L;
+  if ((int)blockIdx.x < A.sblocks) {
+    strip_rows<T, EXACT, kStripBatchNt, kRowResidual>(L, A.S, kAllNodes, blockIdx.x, u, f, d, strip_smem, A.K);
+    return;
+  }
+  const int by = ((int)blockIdx.x - A.sblocks) / A.gx, bx = (int)blockIdx.x - A.sblocks - by * A.gx;
   T c[NT];
   int d0[NT], d1[NT];
 #pragma unroll
   for (int k = 0; k < NT; ++k) {
-    c[k] = L.c[k];
-    d0[k] = L.delta[0][k];
-    d1[k] = L.delta[1][k];
+    c[k] = A.Lp->c[k];
+    d0[k] = A.Lp->delta[0][k];
+    d1[k] = A.Lp->delta[1][k];
   }
-  const int n = L.n;
-  constexpr int lo = PER ? 0 : 1;
-  const int q = blockIdx.x * kBX + threadIdx.x;
+  const int q = bx * kBX + threadIdx.x;
   if (q >= L.cols) return;
-  const int jb = blockIdx.y * (kBY * kRows) + threadIdx.y;
+  const int jb = by * (kBY * kRows) + threadIdx.y;
   // Same L2 prefetch as the half-sweeps: FP32 level-0 residual 120 -> 103 us at 4097^2
   // (order 4); FP64 (bound by the FP64 pipe) unchanged, so it skips it.
   if (sizeof(T) == 4) {
@@ -117,13 +146,10 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_residual_nt(
 #pragma unroll
   for (int r = 0; r < kRows; ++r) {
     const int j = jb + r * kBY;
-    if (j < lo || j >= n) continue;
     const int i = L.kind == kRot ? 2 * q + (j & 1) : q;
-    if (i < lo || i >= n) continue;
+    if (!fast_node_c<PER>(L, i, j)) continue;
     const int64_t at = (int64_t)j * L.pitch + q;
-    const T s = fast_node_c<PER>(L, i, j) ? apply_fast<T, EXACT, NT>(c, (L.kind == kRot && (i & 1)) ? d1 : d0, u, at)
-                                          : apply_at<T, EXACT, 1>(L, u, i, j, at, nullptr);
-    d[at] = rnd(L, Arith<T>::sub(f[at], s));
+    d[at] = rnd(L, Arith<T>::sub(f[at], apply_fast<T, EXACT, NT>(c, (L.kind == kRot && (i & 1)) ? d1 : d0, u, at)));
   }
 }
 
@@ -148,13 +174,22 @@ __device__ __forceinline__ void stage_stencil(const LevelDev<T>& L, StencilSmem<
   __syncthreads();
 }
 
-// U: unroll factor of the term loop (its loads then run ahead of the ordered sum).
-template <typename T, bool EXACT, int U = 4>
+// U: values loaded ahead of the ordered sum of their products (the group flags are
+// uniform over the block, but a branch on them would keep each load behind the sum
+// before it).
+template <typename T, bool EXACT, int U>
 __device__ __forceinline__ T apply_smem(const StencilSmem<T>& sm, int nt, int par, const T* __restrict__ u, int64_t at) {
   const int* dl = sm.d[par];
   RowSum<T, EXACT> acc;
-#pragma unroll U
-  for (int k = 0; k < nt; ++k) acc.add(sm.c[k], u[at + dl[k]], gbit(sm.gm, k));
+  int k = 0;
+  for (; k + U <= nt; k += U) {
+    T x[U];
+#pragma unroll
+    for (int r = 0; r < U; ++r) x[r] = u[at + dl[k + r]];
+#pragma unroll
+    for (int r = 0; r < U; ++r) acc.add(sm.c[k + r], x[r], gbit(sm.gm, k + r));
+  }
+  for (; k < nt; ++k) acc.add(sm.c[k], u[at + dl[k]], gbit(sm.gm, k));
   return acc.value();
 }
 
@@ -171,55 +206,64 @@ struct GenCfg {
 constexpr int kGenDeepRows = 2048;
 
 template <typename T, bool EXACT, bool DEEP>
-__global__ void __launch_bounds__(kBX * kBY, GenCfg<T, DEEP>::min_blocks) k_half_sweep_gen(const LevelDev<T>* __restrict__ Lp, const T* __restrict__ uin,
-                                 const T* __restrict__ f, T* __restrict__ uout, int red) {
-  const LevelDev<T>& L = *Lp;
+__global__ void __launch_bounds__(kBX * kBY, GenCfg<T, DEEP>::min_blocks)
+    k_half_sweep_gen(const __grid_constant__ SweepArgs<T> A, const T* __restrict__ uin, const T* __restrict__ f,
+                     T* __restrict__ uout) {
+  extern __shared__ __align__(16) unsigned char strip_smem[];
+  const LevelGeo<T>& L = A.L;
+  const int red = A.colour;
+  if ((int)blockIdx.x < A.sblocks) {
+    strip_rows<T, EXACT, kStripBatchGen, kRowRelax>(L, A.S, red, blockIdx.x, uin, f, uout, strip_smem, A.K);
+    return;
+  }
+  const int by = ((int)blockIdx.x - A.sblocks) / A.gx, bx = (int)blockIdx.x - A.sblocks - by * A.gx;
   __shared__ StencilSmem<T> sm;
-  stage_stencil(L, sm);
-  int i, j;
+  if (!A.S.all) stage_stencil(*A.Lp, sm);
+  int i, j = by * blockDim.y + threadIdx.y;
+  if (j < L.lo || j >= L.n) return;
   if (L.kind == kAxis) {
-    const int i0 = 2 * (blockIdx.x * kBX + threadIdx.x);
-    j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int lo = L.lo;
-    if (j < lo || j >= L.n || i0 > L.n) return;
+    const int i0 = 2 * (bx * kBX + threadIdx.x);
     i = (((i0 + j) & 1) == red) ? i0 : i0 + 1;
     const int ic = 2 * i0 + 1 - i;
-    if (ic >= lo && ic < L.n) {
+    if (ic >= L.lo && ic < L.n) {
       const int64_t ac = sidx(L, ic, j);
       uout[ac] = uin[ac];
     }
-    if (i < lo || i >= L.n) return;
   } else {
-    if (!thread_node(L, i, j) || !interior(L, i, j)) return;
-    if (is_red(L, i, j) != red) {
+    i = 2 * (bx * kBX + threadIdx.x) + (j & 1);
+    if ((i & 1) != red) {
+      if (i < L.lo || i >= L.n) return;
       const int64_t at = sidx(L, i, j);
       uout[at] = uin[at];
       return;
     }
   }
+  if (A.S.all || !fast_node(L, i, j)) return;  // off the fast rectangle: the octets' node
   const int64_t at = sidx(L, i, j);
-  if (fast_node(L, i, j)) {
-    const T r = Arith<T>::sub(f[at], apply_smem<T, EXACT, GenCfg<T, DEEP>::unroll>(sm, L.nt, L.kind == kRot ? (i & 1) : 0,
-                                                                                 uin, at));
-    const T wd = L.wd;
-    uout[at] = rnd(L, EXACT ? Arith<T>::add(uin[at], Arith<T>::mul(r, wd)) : Arith<T>::fma(r, wd, uin[at]));
-  } else {
-    uout[at] = rnd(L, relax_value<T, EXACT>(L, uin, f, i, j, at));
-  }
+  const T r = Arith<T>::sub(f[at], apply_smem<T, EXACT, GenCfg<T, DEEP>::unroll>(sm, L.nt, L.kind == kRot ? (i & 1) : 0,
+                                                                               uin, at));
+  const T wd = L.wd;
+  uout[at] = rnd(L, EXACT ? Arith<T>::add(uin[at], Arith<T>::mul(r, wd)) : Arith<T>::fma(r, wd, uin[at]));
 }
 
 template <typename T, bool EXACT, bool DEEP>
-__global__ void __launch_bounds__(kBX * kBY, GenCfg<T, DEEP>::min_blocks) k_residual_gen(const LevelDev<T>* __restrict__ Lp, const T* __restrict__ u,
-                               const T* __restrict__ f, T* __restrict__ d) {
-  const LevelDev<T>& L = *Lp;
+__global__ void __launch_bounds__(kBX * kBY, GenCfg<T, DEEP>::min_blocks)
+    k_residual_gen(const __grid_constant__ SweepArgs<T> A, const T* __restrict__ u, const T* __restrict__ f,
+                   T* __restrict__ d) {
+  extern __shared__ __align__(16) unsigned char strip_smem[];
+  const LevelGeo<T>& L = A.L;
+  if ((int)blockIdx.x < A.sblocks) {
+    strip_rows<T, EXACT, kStripBatchGen, kRowResidual>(L, A.S, kAllNodes, blockIdx.x, u, f, d, strip_smem, A.K);
+    return;
+  }
+  const int by = ((int)blockIdx.x - A.sblocks) / A.gx, bx = (int)blockIdx.x - A.sblocks - by * A.gx;
   __shared__ StencilSmem<T> sm;
-  stage_stencil(L, sm);
-  int i, j;
-  if (!thread_node(L, i, j) || !interior(L, i, j)) return;
+  stage_stencil(*A.Lp, sm);
+  const int q = bx * kBX + threadIdx.x, j = by * blockDim.y + threadIdx.y;
+  const int i = L.kind == kRot ? 2 * q + (j & 1) : q;
+  if (!fast_node(L, i, j)) return;
   const int64_t at = sidx(L, i, j);
-  const T s = fast_node(L, i, j) ? apply_smem<T, EXACT, GenCfg<T, DEEP>::unroll>(sm, L.nt, L.kind == kRot ? (i & 1) : 0, u, at)
-                                 : apply_at<T, EXACT>(L, u, i, j, at, nullptr);
-  d[at] = rnd(L, Arith<T>::sub(f[at], s));
+  d[at] = rnd(L, Arith<T>::sub(f[at], apply_smem<T, EXACT, GenCfg<T, DEEP>::unroll>(sm, L.nt, L.kind == kRot ? (i & 1) : 0, u, at)));
 }
 
 // ---- fused red-black sweep on a shared-memory tile ---------------------------
@@ -407,16 +451,16 @@ __host__ __device__ constexpr double rt_w(int tr, int k) {
 // Storage position of lattice node (i, j): in the level's global storage, or in the
 // compact rows x cols layout of the shared-memory tail.
 template <typename T>
-__device__ __forceinline__ int smem_idx(const LevelDev<T>& L, int i, int j) {
+__device__ __forceinline__ int smem_idx(const LevelGeo<T>& L, int i, int j) {
   return j * L.cols + (L.kind == kRot ? (i >> 1) : i);
 }
 struct GlobalIdx {
   template <typename T>
-  __device__ __forceinline__ int64_t operator()(const LevelDev<T>& L, int i, int j) const { return sidx(L, i, j); }
+  __device__ __forceinline__ int64_t operator()(const LevelGeo<T>& L, int i, int j) const { return sidx(L, i, j); }
 };
 struct SmemIdx {
   template <typename T>
-  __device__ __forceinline__ int64_t operator()(const LevelDev<T>& L, int i, int j) const { return smem_idx(L, i, j); }
+  __device__ __forceinline__ int64_t operator()(const LevelGeo<T>& L, int i, int j) const { return smem_idx(L, i, j); }
 };
 
 // Periodic transfers: terms (lattice i, j, weight) on level L wrap modulo L.n, are
@@ -425,7 +469,7 @@ struct SmemIdx {
 // small sums, so the merged weight is exact); then the usual ordered sum.
 constexpr int kMaxTransferTerms = 25;
 template <typename T, bool EXACT, class Idx>
-__device__ __forceinline__ T wrapped_sum(const LevelDev<T>& L, int nt, const int* ti, const int* tj, const T* w,
+__device__ __forceinline__ T wrapped_sum(const LevelGeo<T>& L, int nt, const int* ti, const int* tj, const T* w,
                          const T* __restrict__ x, Idx idx) {
   int64_t pos[kMaxTransferTerms];
   T wt[kMaxTransferTerms];
@@ -457,7 +501,7 @@ __device__ __forceinline__ T wrapped_sum(const LevelDev<T>& L, int nt, const int
 
 // Restriction from a periodic level.
 template <typename T, bool EXACT, int TR, class Idx>
-__device__ __forceinline__ T restrict_wrapped(const LevelDev<T>& Lf, const T* __restrict__ d, int fi, int fj,
+__device__ __forceinline__ T restrict_wrapped(const LevelGeo<T>& Lf, const T* __restrict__ d, int fi, int fj,
                                               Idx idx) {
   constexpr int nt = rt_count(TR);
   int ti[kMaxTransferTerms], tj[kMaxTransferTerms];
@@ -472,7 +516,7 @@ __device__ __forceinline__ T restrict_wrapped(const LevelDev<T>& Lf, const T* __
 }
 
 template <typename T, bool EXACT, int TR, class Idx>
-__device__ __forceinline__ T restrict_sum(const LevelDev<T>& Lf, const T* __restrict__ d, int fi, int fj, Idx idx) {
+__device__ __forceinline__ T restrict_sum(const LevelGeo<T>& Lf, const T* __restrict__ d, int fi, int fj, Idx idx) {
   T s = Arith<T>::mul(T(rt_w(TR, 0)), d[idx(Lf, fi + rt_dx(TR, 0), fj + rt_dy(TR, 0))]);
 #pragma unroll
   for (int k = 1; k < rt_count(TR); ++k)
@@ -484,7 +528,7 @@ __device__ __forceinline__ T restrict_sum(const LevelDev<T>& Lf, const T* __rest
 // are periodic (a compile-time choice, so that the Dirichlet kernels carry none of
 // the wrap-around code).
 template <typename T, bool EXACT, bool PER, class Idx = GlobalIdx>
-__device__ __forceinline__ T restrict_value(const LevelDev<T>& Lf, int transfer, const T* __restrict__ d,
+__device__ __forceinline__ T restrict_value(const LevelGeo<T>& Lf, int transfer, const T* __restrict__ d,
                                             int i, int j, Idx idx = Idx()) {
   // fine-lattice position of the coarse node
   const int fi = transfer == kRbAxisToRot ? i : 2 * i;
@@ -536,7 +580,7 @@ __device__ __forceinline__ int prolong_terms(int transfer, int i, int j, int* ti
 
 // Interpolation from a periodic coarse level.
 template <typename T, bool EXACT, class Idx>
-__device__ __forceinline__ T prolong_wrapped(const LevelDev<T>& Lc, int transfer, const T* __restrict__ vc,
+__device__ __forceinline__ T prolong_wrapped(const LevelGeo<T>& Lc, int transfer, const T* __restrict__ vc,
                                           int i, int j, Idx idx) {
   int ti[4], tj[4];
   T w[4];
@@ -546,7 +590,7 @@ __device__ __forceinline__ T prolong_wrapped(const LevelDev<T>& Lc, int transfer
 
 // Interpolated correction (P v)(i, j) at fine node (i, j) (PER as in restrict_value).
 template <typename T, bool EXACT, bool PER, class Idx = GlobalIdx>
-__device__ __forceinline__ T prolong_value(const LevelDev<T>& Lc, int transfer, const T* __restrict__ vc,
+__device__ __forceinline__ T prolong_value(const LevelGeo<T>& Lc, int transfer, const T* __restrict__ vc,
                                            int i, int j, Idx idx = Idx()) {
   if (PER) return prolong_wrapped<T, EXACT>(Lc, transfer, vc, i, j, idx);
   T e;
@@ -610,7 +654,7 @@ __host__ __device__ constexpr T cubic_r1(int a) {
 // reflection), boundary positions dropped; then as wrapped_sum (ordered by storage
 // position, equal positions merged by exact weight sums).
 template <typename T, bool EXACT, class Idx>
-__device__ __forceinline__ T folded_sum(const LevelDev<T>& L, int nt, const int* ti, const int* tj, const T* w,
+__device__ __forceinline__ T folded_sum(const LevelGeo<T>& L, int nt, const int* ti, const int* tj, const T* w,
                                         const T* __restrict__ x, Idx idx) {
   int64_t pos[kMaxTransferTerms];
   T wt[kMaxTransferTerms];
@@ -648,7 +692,7 @@ __device__ __forceinline__ T folded_sum(const LevelDev<T>& L, int nt, const int*
 }
 
 template <typename T, bool EXACT, bool PER, class Idx>
-__device__ __forceinline__ T edge_sum(const LevelDev<T>& L, int nt, const int* ti, const int* tj, const T* w,
+__device__ __forceinline__ T edge_sum(const LevelGeo<T>& L, int nt, const int* ti, const int* tj, const T* w,
                                       const T* __restrict__ x, Idx idx) {
   if (PER) return wrapped_sum<T, EXACT>(L, nt, ti, tj, w, x, idx);
   return folded_sum<T, EXACT>(L, nt, ti, tj, w, x, idx);
@@ -656,7 +700,7 @@ __device__ __forceinline__ T edge_sum(const LevelDev<T>& L, int nt, const int* t
 
 // Restricted residual at coarse node (i, j) with the cubic adjoint.
 template <typename T, bool EXACT, bool PER, class Idx = GlobalIdx>
-__device__ __forceinline__ T restrict_cubic_value(const LevelDev<T>& Lf, const T* __restrict__ d, int i, int j,
+__device__ __forceinline__ T restrict_cubic_value(const LevelGeo<T>& Lf, const T* __restrict__ d, int i, int j,
                                                   Idx idx = Idx()) {
   const int fi = 2 * i, fj = 2 * j;
   const int lo = PER ? 3 : 4, hi = Lf.n - (PER ? 4 : 4);  // all taps on unknowns, no wrap
@@ -700,7 +744,7 @@ __device__ __forceinline__ int cubic_taps(int i, int* c, T* w) {
 
 // Interpolated correction (P v)(i, j) at fine node (i, j) with cubic interpolation.
 template <typename T, bool EXACT, bool PER, class Idx = GlobalIdx>
-__device__ __forceinline__ T prolong_cubic_value(const LevelDev<T>& Lc, const T* __restrict__ vc, int i, int j,
+__device__ __forceinline__ T prolong_cubic_value(const LevelGeo<T>& Lc, const T* __restrict__ vc, int i, int j,
                                                  Idx idx = Idx()) {
   int cx[4], cy[4];
   T wx[4], wy[4];
@@ -730,7 +774,7 @@ __device__ __forceinline__ T prolong_cubic_value(const LevelDev<T>& Lc, const T*
 
 // Any transfer, boundary kind chosen at run time (tail kernels).
 template <typename T, bool EXACT, class Idx = GlobalIdx>
-__device__ __forceinline__ T restrict_any(const LevelDev<T>& Lf, int transfer, const T* __restrict__ d, int i, int j,
+__device__ __forceinline__ T restrict_any(const LevelGeo<T>& Lf, int transfer, const T* __restrict__ d, int i, int j,
                                           Idx idx = Idx()) {
   if (transfer == kStandardCubic)
     return Lf.per ? restrict_cubic_value<T, EXACT, true>(Lf, d, i, j, idx)
@@ -740,7 +784,7 @@ __device__ __forceinline__ T restrict_any(const LevelDev<T>& Lf, int transfer, c
 }
 
 template <typename T, bool EXACT, class Idx = GlobalIdx>
-__device__ __forceinline__ T prolong_any(const LevelDev<T>& Lc, int transfer, const T* __restrict__ vc, int i, int j,
+__device__ __forceinline__ T prolong_any(const LevelGeo<T>& Lc, int transfer, const T* __restrict__ vc, int i, int j,
                                          Idx idx = Idx()) {
   if (transfer == kStandardCubic)
     return Lc.per ? prolong_cubic_value<T, EXACT, true>(Lc, vc, i, j, idx)
@@ -752,7 +796,7 @@ __device__ __forceinline__ T prolong_any(const LevelDev<T>& Lc, int transfer, co
 // Stores the restricted value v of coarse node (i, j); with tc also the coarse level's
 // first half-sweep from u = 0 (the value k_first_half_zero would write from this f).
 template <typename T>
-__device__ __forceinline__ void store_restricted(const LevelDev<T>& Lc, T* __restrict__ fc, T* __restrict__ tc,
+__device__ __forceinline__ void store_restricted(const LevelGeo<T>& Lc, T* __restrict__ fc, T* __restrict__ tc,
                                                  int i, int j, T v) {
   const int64_t at = sidx(Lc, i, j);
   fc[at] = v;
@@ -922,18 +966,58 @@ __device__ __forceinline__ bool dense_coarse(const DenseCoarse<T>& C, const Leve
   return true;
 }
 
-struct BlockSync {
-  __device__ __forceinline__ bool operator()() const {
-    __syncthreads();
-    return true;
+// The same solve by one block, with d and y kept as contiguous vectors v[0 .. m) and
+// v[m .. 2 m) in shared memory: the values are then broadcasts and every load of G is
+// independent of the others (kDV in flight per row; the index table of unknowns is
+// read once per vector instead of once per product).
+template <typename T, bool EXACT, class IDX>
+__device__ __forceinline__ void dense_coarse_vec(const DenseCoarse<T>& C, const LevelGeo<T>& L, const T* F, T* v, T* U,
+                                                 IDX idx, int tid, int nth) {
+  constexpr int kDV = sizeof(T) == 4 ? 24 : 12;
+  const int m = C.m;
+  T* y = v + m;
+  for (int k = tid; k < m; k += nth) {
+    const int2 q = C.ij[k];
+    v[k] = F[idx(L, q.x, q.y)];
   }
-};
+  __syncthreads();
+  for (int i = tid; i < m; i += nth) {
+    const T* g = C.ga + i;
+    T s = Arith<T>::mul(g[0], v[0]);
+    int k = 1;
+    for (; k + kDV - 1 <= i; k += kDV) {
+      T w[kDV];
+#pragma unroll
+      for (int r = 0; r < kDV; ++r) w[r] = g[(int64_t)(k + r) * m];
+#pragma unroll
+      for (int r = 0; r < kDV; ++r) s = madd<T, EXACT>(s, w[r], v[k + r]);
+    }
+    for (; k <= i; ++k) s = madd<T, EXACT>(s, g[(int64_t)k * m], v[k]);
+    y[i] = s;
+  }
+  __syncthreads();
+  for (int i = tid; i < m; i += nth) {
+    const T* g = C.gb + i;
+    T s = Arith<T>::mul(g[(int64_t)i * m], y[i]);
+    int k = i + 1;
+    for (; k + kDV - 1 < m; k += kDV) {
+      T w[kDV];
+#pragma unroll
+      for (int r = 0; r < kDV; ++r) w[r] = g[(int64_t)(k + r) * m];
+#pragma unroll
+      for (int r = 0; r < kDV; ++r) s = madd<T, EXACT>(s, w[r], y[k + r]);
+    }
+    for (; k < m; ++k) s = madd<T, EXACT>(s, g[(int64_t)k * m], y[k]);
+    const int2 p = C.ij[i];
+    U[idx(L, p.x, p.y)] = s;
+  }
+}
 
 template <typename T, bool EXACT>
-__global__ void __launch_bounds__(1024) k_coarsest_dense(DenseCoarse<T> C, const LevelDev<T>* __restrict__ Lp,
-                                                         const T* __restrict__ f, T* __restrict__ y,
-                                                         T* __restrict__ u) {
-  dense_coarse<T, EXACT>(C, *Lp, f, y, u, GlobalIdx(), (int)threadIdx.x, (int)blockDim.x, BlockSync());
+__global__ void __launch_bounds__(1024) k_coarsest_dense(DenseCoarse<T> C, const __grid_constant__ LevelGeo<T> L,
+                                                         const T* __restrict__ f, T* __restrict__ u) {
+  __shared__ T v[2 * kMaxDense];
+  dense_coarse_vec<T, EXACT>(C, L, f, v, u, GlobalIdx(), (int)threadIdx.x, (int)blockDim.x);
 }
 
 // Block-wide sum of a double (blockDim = kBX * kBY = 256 threads).
@@ -1175,7 +1259,7 @@ constexpr int kTailThreads = 1024;
 
 // Storage element k of a level (row-major over rows x cols) -> lattice node.
 template <typename T>
-__device__ __forceinline__ bool tail_node(const LevelDev<T>& L, int k, int& i, int& j) {
+__device__ __forceinline__ bool tail_node(const LevelGeo<T>& L, int k, int& i, int& j) {
   j = k / L.cols;
   const int q = k - j * L.cols;
   i = L.kind == kRot ? 2 * q + (j & 1) : q;
@@ -1357,8 +1441,8 @@ __global__ void __launch_bounds__(256) k_batch_coarsest_dense(const BatchLevel<T
                                                               const int* __restrict__ active) {
   const BatchLevel<T>& B = E[blockIdx.x];
   if (!active[B.problem]) return;  // uniform over the block
-  dense_coarse<T, EXACT>(B.dense, *B.Lc, B.fc, B.dc, B.uc, GlobalIdx(), (int)threadIdx.x, (int)blockDim.x,
-                         BlockSync());
+  __shared__ T v[2 * kMaxDense];
+  dense_coarse_vec<T, EXACT>(B.dense, *B.Lc, B.fc, v, B.uc, GlobalIdx(), (int)threadIdx.x, (int)blockDim.x);
 }
 
 template <bool EXACT>
@@ -1435,145 +1519,153 @@ __global__ void __launch_bounds__(kBX * kBY)
 
 // ---- shared-memory-resident tail ---------------------------------------------
 // Levels from sm_top down live in one block's shared memory in a compact rows x cols
-// layout; node (i, j) of a level is at j * cols + (rot ? i >> 1 : i). Arithmetic
-// per node is the same as relax_value / apply_at / restrict_value / prolong_value.
-// The interior stencils of the levels held are staged in shared memory too (per level:
-// coefficients, and shared-memory offsets for even and odd i), so that a fast node's
-// terms need no global-memory reads.
-struct TailStencil {
-  template <typename T>
-  static __host__ __device__ __forceinline__ size_t base(int sm_elems) {  // byte offset of the stencil area
+// layout; node (i, j) of a level is at j * cols + (rot ? i >> 1 : i). Operator rows are
+// evaluated by octets of lanes (rows.cuh), sm_octs of them, from class rows that stay in
+// L1 after their first use. Arithmetic per node is the same as relax_value / apply_at /
+// restrict_value / prolong_value.
+//
+// A sweep reads the level's current array A and writes the other one, B: the red phase
+// reads A and writes B's red nodes, the black phase reads B at red and A at black nodes
+// and writes B's black nodes; then the arrays change roles (bit l of `flip`: level l's
+// current array is t). No colour is copied.
+// 512 threads (64 octets, 128 registers): with 1024 the row evaluation spilled in FP64.
+constexpr int kTailSmemThreads = 512;
+template <typename T>
+struct TailSmem {
+  static __host__ __device__ __forceinline__ size_t stage(int sm_elems) {  // byte offset of the octets' staging
     return ((size_t)sm_elems * sizeof(T) + 15) & ~(size_t)15;
   }
 };
 
-template <typename T, bool EXACT>
-__device__ __forceinline__ T smem_apply(const LevelDev<T>& L, const T* u, int i, int j, T* wd, const T* __restrict__ cs,
-                                        const int* __restrict__ os2) {
-  RowSum<T, EXACT> acc;
-  if (fast_node(L, i, j)) {
-    const int* os = os2 + (L.kind == kRot ? (i & 1) : 0) * kMaxTerms;
-    const int e = smem_idx(L, i, j);
-#pragma unroll 8
-    for (int k = 0; k < L.nt; ++k) acc.add(cs[k], u[e + os[k]], gbit(L.gmask, k));
-    if (wd) *wd = L.wd;
-  } else {
-    const int cl = class_of(L, i, j);
-    const int2 ce = L.cls[cl];
-    const ClassTerm<T>* tt = L.terms + ce.x;
-#pragma unroll 4
-    for (int k = 0; k < ce.y; ++k) {
-      const Term<T> t = load_term(tt + k);
-      acc.add(t.c, u[smem_idx(L, i + t.dx, j + t.dy)], t.start);
-    }
-    if (wd) *wd = L.cls_wd[cl];
+// All unknowns of one colour (or all) of a level, one slot each (as make_strips with
+// `all`): slots, and slot -> node.
+template <typename T>
+struct LevelSlots {
+  int lo, hi, rstep, cstep, first, w, total, colour, kind;
+  __device__ __forceinline__ LevelSlots(const LevelGeo<T>& L, int c) : lo(L.lo), hi(L.n - 1), colour(c), kind(L.kind) {
+    rstep = (kind == kRot && c != kAllNodes) ? 2 : 1;
+    cstep = (kind == kAxis && c == kAllNodes) ? 1 : 2;
+    first = rstep == 2 ? lo + ((lo ^ c) & 1) : lo;
+    w = (hi - lo) / cstep + 1;
+    total = (first > hi ? 0 : (hi - first) / rstep + 1) * w;
   }
-  return acc.value();
-}
+  __device__ __forceinline__ bool node(int slot, int& i, int& j) const {
+    if (slot >= total) return false;
+    const int r = slot / w, s = slot - r * w;
+    j = first + r * rstep;
+    if (cstep == 1) {
+      i = lo + s;
+    } else {
+      const int par = kind == kRot ? (j & 1) : ((j ^ colour) & 1);
+      i = lo + ((lo ^ par) & 1) + 2 * s;
+    }
+    return i <= hi;
+  }
+};
 
 template <typename T, bool EXACT>
-__global__ void __launch_bounds__(kTailThreads, 1)
+__global__ void __launch_bounds__(kTailSmemThreads, 1)
     k_tail_smem(const TailDesc<T>* __restrict__ D, const int4* __restrict__ prog, int nops) {
   extern __shared__ __align__(16) unsigned char tail_smem[];
+  __shared__ LevelGeo<T> geo[kTailMaxLevels];
   T* sm = reinterpret_cast<T*>(tail_smem);
-  const int tid = threadIdx.x;
-  const int top = D->sm_top;
-  for (int k = tid; k < D->sm_elems; k += kTailThreads) sm[k] = T(0);
-  // interior stencils of the levels held: coefficients [level][kMaxTerms], offsets
-  // [level][parity][kMaxTerms]
-  const int nst = D->nlev - top;
-  T* stc = reinterpret_cast<T*>(tail_smem + TailStencil::base<T>(D->sm_elems));
-  int* sto = reinterpret_cast<int*>(stc + nst * kMaxTerms);
-  for (int x = tid; x < nst * kMaxTerms; x += kTailThreads) {
-    const int l = top + x / kMaxTerms, k = x - (x / kMaxTerms) * kMaxTerms;
-    const LevelDev<T>& L = *D->L[l];
-    if (k < L.nt) {
-      stc[x] = L.c[k];
-      sto[2 * (l - top) * kMaxTerms + k] = L.sdy[k] * L.cols + L.sdx[0][k];
-      sto[(2 * (l - top) + 1) * kMaxTerms + k] = L.sdy[k] * L.cols + L.sdx[1][k];
-    }
-  }
+  const int tid = threadIdx.x, lane = tid & 31, oct = tid >> 3;
+  const int top = D->sm_top, nocts = D->sm_octs, K = D->sm_K;
+  unsigned char* stage = tail_smem + TailSmem<T>::stage(D->sm_elems) + oct * oct_bytes<T>(K);
+  for (int k = tid; k < D->sm_elems; k += kTailSmemThreads) sm[k] = T(0);
+  for (int l = top + tid; l < D->nlev; l += kTailSmemThreads) geo[l] = *D->L[l];
   __syncthreads();
   {  // top level: u and f from global memory
-    const LevelDev<T>& L = *D->L[top];
-    for (int k = tid; k < L.rows * L.cols; k += kTailThreads) {
+    const LevelGeo<T>& L = geo[top];
+    for (int k = tid; k < L.rows * L.cols; k += kTailSmemThreads) {
       const int j = k / L.cols, q = k - j * L.cols;
       sm[D->sm_u[top] + k] = D->u[top][(int64_t)j * L.pitch + q];
       sm[D->sm_f[top] + k] = D->f[top][(int64_t)j * L.pitch + q];
     }
   }
   __syncthreads();
+  uint64_t flip = 0;
+  auto cur = [&](int l) { return ((flip >> l) & 1) ? D->sm_t[l] : D->sm_u[l]; };
+  auto oth = [&](int l) { return ((flip >> l) & 1) ? D->sm_u[l] : D->sm_t[l]; };
+  // fin(k, i, j, (L u)(i, j), cl) in the first lane of the octet of every node of colour
+  // c; a term at a red node reads the array at offset `ra`, at a black one `ba`
+  auto rows = [&](int l, int c, int ra, int ba, auto fin) {
+    const LevelGeo<T>& L = geo[l];
+    const LevelSlots<T> S(L, c);
+    const int cols = L.cols, rot = L.kind == kRot;
+    auto pos = [=](int i, int j) {
+      const int red = rot ? (i & 1) : ((i + j) & 1);
+      return (red ? ra : ba) + j * cols + (rot ? (i >> 1) : i);
+    };
+    for (int s0 = 0; s0 < S.total; s0 += nocts) {
+      if (oct >= nocts || s0 + (oct & ~3) >= S.total) break;  // uniform over a warp
+      int i = 0, j = 0;
+      const bool on = S.node(s0 + oct, i, j);
+      const int cl = on ? class_of(L, i, j) : 0;
+      const T v = octet_row<T, EXACT, 6>(L, sm, on, i, j, cl, stage, K, pos);
+      if (on && (lane & 7) == 0) fin(smem_idx(L, i, j), v, cl);
+    }
+  };
   for (int p = 0; p < nops; ++p) {
     const int4 op = prog[p];
     const int l = op.y;
-    const LevelDev<T>& L = *D->L[l];
+    const LevelGeo<T>& L = geo[l];
     const int total = L.rows * L.cols;
-    T* U = sm + D->sm_u[l];
-    T* Tb = sm + D->sm_t[l];
-    T* F = sm + D->sm_f[l];
-    const T* cs = stc + (l - top) * kMaxTerms;
-    const int* os2 = sto + 2 * (l - top) * kMaxTerms;
+    const T* F = sm + D->sm_f[l];
     int i, j;
     if (op.x == kOpZero) {
-      for (int k = tid; k < total; k += kTailThreads) U[k] = T(0);
+      T* U = sm + cur(l);
+      for (int k = tid; k < total; k += kTailSmemThreads) U[k] = T(0);
     } else if (op.x == kOpSmooth) {
+      const int ca = cur(l), cb = oth(l);
+      auto relax = [&](int k, T v, int cl) {
+        const T r = Arith<T>::sub(F[k], v), wd = L.cls_wd[cl];
+        const T x = sm[ca + k];
+        sm[cb + k] = EXACT ? Arith<T>::add(x, Arith<T>::mul(r, wd)) : Arith<T>::fma(r, wd, x);
+      };
       if (D->smoother == 0) {
-        for (int half = 1; half >= 0; --half) {
-          const T* src = half ? U : Tb;
-          T* dst = half ? Tb : U;
-          for (int k = tid; k < total; k += kTailThreads) {
+        if (op.z) {  // first half-sweep from u = 0 (op.z: the array was not zeroed)
+          for (int k = tid; k < total; k += kTailSmemThreads) {
             if (!tail_node(L, k, i, j)) continue;
-            if (op.z && half) {  // first half-sweep from u = 0 (op.z: U not zeroed)
-              dst[k] = is_red(L, i, j) ? relax_from_zero(F[k], node_wd(L, i, j)) : T(0);
-            } else if (is_red(L, i, j) == half) {
-              T wd;
-              const T r = Arith<T>::sub(F[k], smem_apply<T, EXACT>(L, src, i, j, &wd, cs, os2));
-              dst[k] = EXACT ? Arith<T>::add(src[k], Arith<T>::mul(r, wd)) : Arith<T>::fma(r, wd, src[k]);
-            } else {
-              dst[k] = src[k];
-            }
+            if (is_red(L, i, j)) sm[cb + k] = relax_from_zero(F[k], node_wd(L, i, j));
+            else sm[ca + k] = T(0);
           }
-          __syncthreads();
-        }
-      } else {
-        for (int k = tid; k < total; k += kTailThreads) {
-          if (!tail_node(L, k, i, j)) continue;
-          T wd;
-          const T r = Arith<T>::sub(F[k], smem_apply<T, EXACT>(L, U, i, j, &wd, cs, os2));
-          Tb[k] = EXACT ? Arith<T>::add(U[k], Arith<T>::mul(r, wd)) : Arith<T>::fma(r, wd, U[k]);
+        } else {
+          rows(l, kRedNodes, ca, ca, relax);
         }
         __syncthreads();
-        for (int k = tid; k < total; k += kTailThreads) {
-          if (!tail_node(L, k, i, j)) continue;
-          U[k] = Tb[k];
-        }
+        rows(l, kBlackNodes, cb, ca, relax);
+      } else {
+        rows(l, kAllNodes, ca, ca, relax);
       }
+      flip ^= 1ull << l;
     } else if (op.x == kOpResRestrict) {
       T* Dd = sm + D->sm_d[l];
-      for (int k = tid; k < total; k += kTailThreads) {
-        if (!tail_node(L, k, i, j)) continue;
-        Dd[k] = Arith<T>::sub(F[k], smem_apply<T, EXACT>(L, U, i, j, nullptr, cs, os2));
-      }
+      const int c = cur(l);
+      rows(l, kAllNodes, c, c, [&](int k, T v, int) { Dd[k] = Arith<T>::sub(F[k], v); });
       __syncthreads();
-      const LevelDev<T>& Lc = *D->L[l + 1];
+      const LevelGeo<T>& Lc = geo[l + 1];
       T* Fc = sm + D->sm_f[l + 1];
       const int tr = D->transfer[l];
-      for (int k = tid; k < Lc.rows * Lc.cols; k += kTailThreads) {
+      for (int k = tid; k < Lc.rows * Lc.cols; k += kTailSmemThreads) {
         if (!tail_node(Lc, k, i, j)) continue;
         Fc[k] = restrict_any<T, EXACT>(L, tr, Dd, i, j, SmemIdx());
       }
     } else if (op.x == kOpCoarsest) {
+      T* U = sm + cur(l);
       if (D->dense.m > 0) {
-        dense_coarse<T, EXACT>(D->dense, L, F, sm + D->sm_d[l], U, SmemIdx(), tid, kTailThreads, BlockSync());
+        T* fv = reinterpret_cast<T*>(tail_smem + TailSmem<T>::stage(D->sm_elems));
+        dense_coarse_vec<T, EXACT>(D->dense, L, F, fv, U, SmemIdx(), tid, kTailSmemThreads);
       } else if (tid == 0) {
         const int c = D->coarsest_zero ? smem_idx(L, 0, 0) : smem_idx(L, 1, 1);
         U[c] = D->coarsest_zero ? T(0) : Arith<T>::div(F[c], D->coarsest_a);
       }
     } else {  // kOpProlong
-      const LevelDev<T>& Lc = *D->L[l + 1];
-      const T* V = sm + D->sm_u[l + 1];
+      const LevelGeo<T>& Lc = geo[l + 1];
+      const T* V = sm + cur(l + 1);
+      T* U = sm + cur(l);
       const int tr = D->transfer[l];
-      for (int k = tid; k < total; k += kTailThreads) {
+      for (int k = tid; k < total; k += kTailSmemThreads) {
         if (!tail_node(L, k, i, j)) continue;
         const T e = prolong_any<T, EXACT>(Lc, tr, V, i, j, SmemIdx());
         U[k] = Arith<T>::add(U[k], e);
@@ -1582,11 +1674,12 @@ __global__ void __launch_bounds__(kTailThreads, 1)
     __syncthreads();
   }
   {  // top level: u back to global memory (interior nodes)
-    const LevelDev<T>& L = *D->L[top];
-    for (int k = tid; k < L.rows * L.cols; k += kTailThreads) {
+    const LevelGeo<T>& L = geo[top];
+    const int c = cur(top);
+    for (int k = tid; k < L.rows * L.cols; k += kTailSmemThreads) {
       int i, j;
       if (!tail_node(L, k, i, j)) continue;
-      D->u[top][(int64_t)j * L.pitch + (k - j * L.cols)] = sm[D->sm_u[top] + k];
+      D->u[top][(int64_t)j * L.pitch + (k - j * L.cols)] = sm[c + k];
     }
   }
 }
@@ -1645,19 +1738,50 @@ int gen_block_rows(const LevelDev<T>& L, unsigned gx) {
   return by;
 }
 
+// Whether every node of a launch goes to the octets (rows.cuh), the fast ones too: small
+// levels, where their shorter chains beat one thread per node as long as the octets' warps
+// leave room on the FP64 units (kOctetWarpsPerUnit warps to each of an SM's four).
+constexpr int kOctetWarpsPerUnit = 2;
+template <typename T>
+bool all_octets(const LevelGeo<T>& L, int colour) {
+  const int64_t nodes = (int64_t)(L.n - L.lo) * (L.n - L.lo) / ((L.kind == kRot ? 2 : 1) * (colour == kAllNodes ? 1 : 2));
+  return nodes <= (int64_t)kOctetWarpsPerUnit * 4 * 4 * sm_count();
+}
+
+// Launch arguments of a half-sweep (colour red or black) or residual (all nodes): `wx` fast
+// nodes' columns of blocks, `rows` storage rows per block of `by` warps.
+template <typename T>
+SweepArgs<T> sweep_args(const LevelPair<T>& L, int colour, int gx, int rows, int by, dim3& grid, size_t& smem) {
+  SweepArgs<T> A;
+  A.L = L.h;
+  A.Lp = L.d;
+  A.S = make_strips<T>(L.h, colour, all_octets<T>(L.h, colour));
+  A.colour = colour;
+  A.K = oct_slots(L.h.maxcnt);
+  A.gx = gx;
+  A.sblocks = (A.S.total + 4 * by - 1) / (4 * by);
+  const int gy = (L.h.rows + rows - 1) / rows;
+  // a residual with no fast nodes needs no other blocks (a half-sweep's copy the other colour)
+  grid = dim3(A.sblocks + (A.S.all && colour == kAllNodes ? 0 : gx * gy));
+  smem = A.sblocks > 0 ? 4 * by * oct_bytes<T>(A.K) : 0;
+  return A;
+}
+
 template <typename T, int NT>
 cudaError_t launch_half_sweep_nt(const LevelPair<T>& L, bool exact, const T* uin, const T* f, T* uout, int red,
                                  cudaStream_t s) {
-  dim3 g = grid_of(L.h);
-  if (L.h.kind == kAxis) g.x = ((L.h.n + 2) / 2 + kBX - 1) / kBX;  // pairs (2p, 2p+1), 2p <= n
-  g.y = (L.h.rows + kBY * RowsPer<T>::value - 1) / (kBY * RowsPer<T>::value);
+  int gx = (L.h.cols + kBX - 1) / kBX;
+  if (L.h.kind == kAxis) gx = ((L.h.n + 2) / 2 + kBX - 1) / kBX;  // pairs (2p, 2p+1), 2p <= n
+  dim3 g;
+  size_t sm;
+  const SweepArgs<T> A = sweep_args(L, red, gx, kBY * RowsPer<T>::value, kBY, g, sm);
   const dim3 b(kBX, kBY);
   if (L.h.per) {
-    if (exact) k_half_sweep_nt<T, true, NT, true><<<g, b, 0, s>>>(L.d, uin, f, uout, red);
-    else k_half_sweep_nt<T, false, NT, true><<<g, b, 0, s>>>(L.d, uin, f, uout, red);
+    if (exact) k_half_sweep_nt<T, true, NT, true><<<g, b, sm, s>>>(A, uin, f, uout);
+    else k_half_sweep_nt<T, false, NT, true><<<g, b, sm, s>>>(A, uin, f, uout);
   } else {
-    if (exact) k_half_sweep_nt<T, true, NT, false><<<g, b, 0, s>>>(L.d, uin, f, uout, red);
-    else k_half_sweep_nt<T, false, NT, false><<<g, b, 0, s>>>(L.d, uin, f, uout, red);
+    if (exact) k_half_sweep_nt<T, true, NT, false><<<g, b, sm, s>>>(A, uin, f, uout);
+    else k_half_sweep_nt<T, false, NT, false><<<g, b, sm, s>>>(A, uin, f, uout);
   }
   return cudaGetLastError();
 }
@@ -1668,17 +1792,20 @@ cudaError_t launch_half_sweep(const LevelPair<T>& L, bool exact, const T* uin, c
   const int ntf = fast_nt(L.h);
   if (ntf == 5) return launch_half_sweep_nt<T, 5>(L, exact, uin, f, uout, red, s);
   if (ntf == 9) return launch_half_sweep_nt<T, 9>(L, exact, uin, f, uout, red, s);
-  dim3 g = grid_of(L.h);
-  if (L.h.kind == kAxis) g.x = ((L.h.n + 2) / 2 + kBX - 1) / kBX;  // pairs (2p, 2p+1), 2p <= n
-  const int by = gen_block_rows(L.h, g.x);
-  g.y = (L.h.rows + by - 1) / by;
+  int gx = (L.h.cols + kBX - 1) / kBX;
+  if (L.h.kind == kAxis) gx = ((L.h.n + 2) / 2 + kBX - 1) / kBX;  // pairs (2p, 2p+1), 2p <= n
+  const int by = gen_block_rows(L.h, gx);
+  dim3 g;
+  size_t sm;
+  const SweepArgs<T> A = sweep_args(L, red, gx, by, by, g, sm);
+  const dim3 b(kBX, by);
   const bool deep = sizeof(T) == 4 && L.h.rows < kGenDeepRows;
   if (deep) {
-    if (exact) k_half_sweep_gen<T, true, true><<<g, dim3(kBX, by), 0, s>>>(L.d, uin, f, uout, red);
-    else k_half_sweep_gen<T, false, true><<<g, dim3(kBX, by), 0, s>>>(L.d, uin, f, uout, red);
+    if (exact) k_half_sweep_gen<T, true, true><<<g, b, sm, s>>>(A, uin, f, uout);
+    else k_half_sweep_gen<T, false, true><<<g, b, sm, s>>>(A, uin, f, uout);
   } else {
-    if (exact) k_half_sweep_gen<T, true, false><<<g, dim3(kBX, by), 0, s>>>(L.d, uin, f, uout, red);
-    else k_half_sweep_gen<T, false, false><<<g, dim3(kBX, by), 0, s>>>(L.d, uin, f, uout, red);
+    if (exact) k_half_sweep_gen<T, true, false><<<g, b, sm, s>>>(A, uin, f, uout);
+    else k_half_sweep_gen<T, false, false><<<g, b, sm, s>>>(A, uin, f, uout);
   }
   return cudaGetLastError();
 }
@@ -1729,15 +1856,17 @@ cudaError_t launch_apply(const LevelPair<T>& L, bool exact, const T* u, T* out, 
 
 template <typename T, int NT>
 cudaError_t launch_residual_nt(const LevelPair<T>& L, bool exact, const T* u, const T* f, T* d, cudaStream_t s) {
-  dim3 g = grid_of(L.h);
-  g.y = (L.h.rows + kBY * RowsPer<T>::value - 1) / (kBY * RowsPer<T>::value);
+  dim3 g;
+  size_t sm;
+  const SweepArgs<T> A =
+      sweep_args(L, kAllNodes, (L.h.cols + kBX - 1) / kBX, kBY * RowsPer<T>::value, kBY, g, sm);
   const dim3 b(kBX, kBY);
   if (L.h.per) {
-    if (exact) k_residual_nt<T, true, NT, true><<<g, b, 0, s>>>(L.d, u, f, d);
-    else k_residual_nt<T, false, NT, true><<<g, b, 0, s>>>(L.d, u, f, d);
+    if (exact) k_residual_nt<T, true, NT, true><<<g, b, sm, s>>>(A, u, f, d);
+    else k_residual_nt<T, false, NT, true><<<g, b, sm, s>>>(A, u, f, d);
   } else {
-    if (exact) k_residual_nt<T, true, NT, false><<<g, b, 0, s>>>(L.d, u, f, d);
-    else k_residual_nt<T, false, NT, false><<<g, b, 0, s>>>(L.d, u, f, d);
+    if (exact) k_residual_nt<T, true, NT, false><<<g, b, sm, s>>>(A, u, f, d);
+    else k_residual_nt<T, false, NT, false><<<g, b, sm, s>>>(A, u, f, d);
   }
   return cudaGetLastError();
 }
@@ -1748,16 +1877,19 @@ cudaError_t launch_residual(const LevelPair<T>& L, bool exact, const T* u, const
   const int ntf = fast_nt(L.h);
   if (ntf == 5) return launch_residual_nt<T, 5>(L, exact, u, f, d, s);
   if (ntf == 9) return launch_residual_nt<T, 9>(L, exact, u, f, d, s);
-  dim3 g = grid_of(L.h);
-  const int by = gen_block_rows(L.h, g.x);
-  g.y = (L.h.rows + by - 1) / by;
+  const int gx = (L.h.cols + kBX - 1) / kBX;
+  const int by = gen_block_rows(L.h, gx);
+  dim3 g;
+  size_t sm;
+  const SweepArgs<T> A = sweep_args(L, kAllNodes, gx, by, by, g, sm);
+  const dim3 b(kBX, by);
   const bool deep = sizeof(T) == 4 && L.h.rows < kGenDeepRows;
   if (deep) {
-    if (exact) k_residual_gen<T, true, true><<<g, dim3(kBX, by), 0, s>>>(L.d, u, f, d);
-    else k_residual_gen<T, false, true><<<g, dim3(kBX, by), 0, s>>>(L.d, u, f, d);
+    if (exact) k_residual_gen<T, true, true><<<g, b, sm, s>>>(A, u, f, d);
+    else k_residual_gen<T, false, true><<<g, b, sm, s>>>(A, u, f, d);
   } else {
-    if (exact) k_residual_gen<T, true, false><<<g, dim3(kBX, by), 0, s>>>(L.d, u, f, d);
-    else k_residual_gen<T, false, false><<<g, dim3(kBX, by), 0, s>>>(L.d, u, f, d);
+    if (exact) k_residual_gen<T, true, false><<<g, b, sm, s>>>(A, u, f, d);
+    else k_residual_gen<T, false, false><<<g, b, sm, s>>>(A, u, f, d);
   }
   return cudaGetLastError();
 }
@@ -1836,11 +1968,11 @@ cudaError_t launch_prolong_add(const LevelPair<T>& Lf, const LevelPair<T>& Lc, i
 }
 
 template <typename T>
-cudaError_t launch_coarsest_dense(const DenseCoarse<T>& C, const LevelPair<T>& L, bool exact, const T* f, T* y, T* u,
+cudaError_t launch_coarsest_dense(const DenseCoarse<T>& C, const LevelPair<T>& L, bool exact, const T* f, T* u,
                                   cudaStream_t s) {
   const int threads = std::min(1024, (C.m + 31) / 32 * 32);
-  if (exact) k_coarsest_dense<T, true><<<1, threads, 0, s>>>(C, L.d, f, y, u);
-  else k_coarsest_dense<T, false><<<1, threads, 0, s>>>(C, L.d, f, y, u);
+  if (exact) k_coarsest_dense<T, true><<<1, threads, 0, s>>>(C, L.h, f, u);
+  else k_coarsest_dense<T, false><<<1, threads, 0, s>>>(C, L.h, f, u);
   return cudaGetLastError();
 }
 
@@ -2068,19 +2200,25 @@ cudaError_t launch_batch_ir_update(const BatchLevel<double>* entries, const int*
 }
 
 template <typename T>
-size_t tail_smem_bytes(int sm_elems, int nst) {
-  return TailStencil::base<T>(sm_elems) + (size_t)nst * kMaxTerms * (sizeof(T) + 2 * sizeof(int));
+TailSmemPlan tail_smem_plan(int sm_elems, int maxcnt, int dense_m) {
+  TailSmemPlan P;
+  P.K = oct_slots(maxcnt);
+  const size_t base = TailSmem<T>::stage(sm_elems), per_warp = 4 * oct_bytes<T>(P.K);
+  const size_t room = base < kTailSmemMaxBytes ? kTailSmemMaxBytes - base : 0;
+  const size_t warps = std::min<size_t>(kTailSmemThreads / 32, room / per_warp);
+  P.octs = 4 * (int)warps;
+  P.bytes = base + std::max(warps * per_warp, 2 * (size_t)dense_m * sizeof(T));
+  if (warps == 0 || P.bytes > kTailSmemMaxBytes) P.octs = 0;
+  return P;
 }
 
 template <typename T>
-cudaError_t launch_tail_smem(const TailDesc<T>* desc, int sm_elems, int nst, const int4* prog, int nops, bool exact,
+cudaError_t launch_tail_smem(const TailDesc<T>* desc, size_t bytes, const int4* prog, int nops, bool exact,
                              cudaStream_t s) {
-  const size_t bytes = tail_smem_bytes<T>(sm_elems, nst);
-  if (bytes > kTailSmemMaxBytes) return cudaErrorInvalidValue;
   const void* fn = exact ? (const void*)k_tail_smem<T, true> : (const void*)k_tail_smem<T, false>;
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (exact) k_tail_smem<T, true><<<1, kTailThreads, bytes, s>>>(desc, prog, nops);
-  else k_tail_smem<T, false><<<1, kTailThreads, bytes, s>>>(desc, prog, nops);
+  if (exact) k_tail_smem<T, true><<<1, kTailSmemThreads, bytes, s>>>(desc, prog, nops);
+  else k_tail_smem<T, false><<<1, kTailSmemThreads, bytes, s>>>(desc, prog, nops);
   return cudaGetLastError();
 }
 
@@ -2098,8 +2236,8 @@ cudaError_t launch_tail_smem(const TailDesc<T>* desc, int sm_elems, int nst, con
                                              const T*, cudaStream_t, const T*);                       \
   template cudaError_t launch_sweep_fused<T>(const LevelPair<T>&, bool, const T*, const T*, T*, cudaStream_t); \
   template cudaError_t launch_coarsest<T>(int64_t, T, int, const T*, T*, cudaStream_t);                    \
-  template cudaError_t launch_coarsest_dense<T>(const DenseCoarse<T>&, const LevelPair<T>&, bool, const T*, T*, T*, \
-                                                cudaStream_t);                                                     \
+  template cudaError_t launch_coarsest_dense<T>(const DenseCoarse<T>&, const LevelPair<T>&, bool, const T*, T*, \
+                                                cudaStream_t);                                                 \
   template int resnorm_blocks<T>(const LevelPair<T>&);                                                \
   template cudaError_t launch_resnorm<T>(const LevelPair<T>&, bool, const T*, const T*, double*,     \
                                          double*, cudaStream_t);                                      \
@@ -2112,8 +2250,8 @@ cudaError_t launch_tail_smem(const TailDesc<T>* desc, int sm_elems, int nst, con
   template cudaError_t launch_batch_step<T>(int, const BatchLevel<T>*, const int*, int, int, int, const int*, bool, \
                                             cudaStream_t);                                             \
   template int tail_ctas<T>(bool);                                                                    \
-  template cudaError_t launch_tail_smem<T>(const TailDesc<T>*, int, int, const int4*, int, bool, cudaStream_t); \
-  template size_t tail_smem_bytes<T>(int, int);                                                       \
+  template cudaError_t launch_tail_smem<T>(const TailDesc<T>*, size_t, const int4*, int, bool, cudaStream_t); \
+  template TailSmemPlan tail_smem_plan<T>(int, int, int);                                             \
   template cudaError_t launch_tail<T>(int, const TailDesc<T>*, const int4*, int, bool, cudaStream_t);
 
 NSMG_INSTANTIATE(double)

@@ -50,10 +50,10 @@ struct DenseCoarse {
   const int2* ij;  // lattice coordinates (i, j) of unknown k, row-major (j, then i)
   int32_t m;       // unknowns; 0: one unknown, solved by the division
 };
-// Dense coarsest solve on level L's storage: u = G^T (G f), y (the level's d array)
-// holds G f in between. One block.
+constexpr int kMaxDense = 1024;  // largest m
+// Dense coarsest solve on level L's storage: u = G^T (G f). One block.
 template <typename T>
-cudaError_t launch_coarsest_dense(const DenseCoarse<T>& C, const LevelPair<T>& L, bool exact, const T* f, T* y, T* u,
+cudaError_t launch_coarsest_dense(const DenseCoarse<T>& C, const LevelPair<T>& L, bool exact, const T* f, T* u,
                                   cudaStream_t s);
 
 // Sum of squares of d = f - L u over interior nodes of an axis level, in FP64:
@@ -119,19 +119,25 @@ struct TailDesc {
   int32_t sm_u[kTailMaxLevels], sm_t[kTailMaxLevels], sm_f[kTailMaxLevels], sm_d[kTailMaxLevels];
   int32_t sm_top;     // first level held (the sub-cycle's top level)
   int32_t sm_elems;   // shared-memory elements of the level arrays
+  int32_t sm_octs, sm_K;  // octets at work and values staged by each (TailSmemPlan)
   int32_t nlev;       // levels of the hierarchy (those from sm_top on are held)
 };
 
 // The same op list, with every level from sm_top down held in one block's shared
 // memory (u and f of the top level are loaded at start, u written back at the end).
 template <typename T>
-cudaError_t launch_tail_smem(const TailDesc<T>* desc, int sm_elems, int nst, const int4* prog, int nops, bool exact,
+cudaError_t launch_tail_smem(const TailDesc<T>* desc, size_t bytes, const int4* prog, int nops, bool exact,
                              cudaStream_t s);
-// Dynamic shared memory of the shared-memory tail: the level arrays (sm_elems values)
-// and the interior stencils of its nst levels; at most kTailSmemMaxBytes.
+// Shared memory of the shared-memory tail: the level arrays (sm_elems values), then the
+// staging of as many octets as fit (rows of up to maxcnt terms), which the dense coarsest
+// solve (dense_m unknowns) reuses. octs = 0: does not fit kTailSmemMaxBytes.
+struct TailSmemPlan {
+  int octs = 0, K = 0;
+  size_t bytes = 0;
+};
 template <typename T>
-size_t tail_smem_bytes(int sm_elems, int nst);
-constexpr size_t kTailSmemMaxBytes = 227 * 1024;
+TailSmemPlan tail_smem_plan(int sm_elems, int maxcnt, int dense_m);
+constexpr size_t kTailSmemMaxBytes = 220 * 1024;  // leaves room for the kernel's static arrays
 
 // Run `nops` ops (x = TailOp, y = level) in order inside one thread-block cluster of
 // `ctas` CTAs, with a cluster barrier after each phase. Op semantics match the

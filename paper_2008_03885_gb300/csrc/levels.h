@@ -47,19 +47,15 @@ struct __align__(16) ClassTerm {
 //   small levels: cx = i, cy = j (table (n+1) x (n+1));
 //   otherwise: cx = i for i < rx, 2 rx - (n - per - i) for i > n - per - rx, rx in
 //   between (single coordinates at both edges, so every class has one term list).
+// The scalars and table pointers of a level, small enough to pass to a kernel by value
+// (a kernel that reads them through a device pointer first waits for that load).
 template <typename T>
-struct LevelDev {
+struct LevelGeo {
   int32_t kind, n, rows, cols, pitch;
   int32_t nt, rx, ry;
   int32_t small, clsw;
+  int32_t maxcnt;             // terms of the longest class row
   T wd;                       // omega / a_pp at fast nodes
-  T c[kMaxTerms];             // fast-node coefficients, in evaluation order: groups of equal
-                              // coefficient (ordered by their first term in (dy, dx) order),
-                              // each group's terms in (dy, dx) order
-  uint32_t gmask[kMaxTerms / 32];  // bit k: fast term k starts a group
-  int32_t delta[2][kMaxTerms];  // storage offsets of the fast terms for i even / odd
-  int32_t sdx[2][kMaxTerms];    // storage-column shift of the fast terms for i even / odd
-  int32_t sdy[kMaxTerms];       // row shift of the fast terms
   const int2* cls;            // per class: (first term, term count)
   const T* cls_wd;            // per class: omega / a_pp
   const ClassTerm<T>* terms;  // merged terms of every class
@@ -67,6 +63,19 @@ struct LevelDev {
   int32_t per;   // 1: periodic level (see above)
   int32_t lo;    // first unknown index: 1 - per
   int32_t fxe, fye;  // last fast-node i and j: n - per - rx, n - per - ry
+  int32_t bdata;     // level 0 with Dirichlet data g: fast rows read the boundary entries,
+                     // which class rows drop
+};
+
+template <typename T>
+struct LevelDev : LevelGeo<T> {
+  T c[kMaxTerms];             // fast-node coefficients, in evaluation order: groups of equal
+                              // coefficient (ordered by their first term in (dy, dx) order),
+                              // each group's terms in (dy, dx) order
+  uint32_t gmask[kMaxTerms / 32];  // bit k: fast term k starts a group
+  int32_t delta[2][kMaxTerms];  // storage offsets of the fast terms for i even / odd
+  int32_t sdx[2][kMaxTerms];    // storage-column shift of the fast terms for i even / odd
+  int32_t sdy[kMaxTerms];       // row shift of the fast terms
 };
 
 }  // namespace nsmg
