@@ -71,6 +71,17 @@ __device__ __forceinline__ Term<T> load_term(const ClassTerm<T>* p) {
 // rather than DRAM (more bytes in flight than the registers of a thread allow).
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
+// Programmatic dependent launch. A kernel launched with the attribute (launch_pdl in
+// kernels.cu) may start once every block of the kernel before it has called pdl_trigger or
+// ended; until pdl_wait returns (the kernel before it complete, its writes visible) it may
+// read only what no kernel writes: its arguments and the level tables. Every thread of
+// such a kernel calls pdl_wait, also those with no node, so that its own completion implies
+// that of all kernels before it. Without the attribute both are no-ops. The arrays that
+// kernels write must not be `const __restrict__` arguments of such a kernel: the compiler
+// takes those for constant while the kernel runs and may load them before the wait.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // s + c * x in the chosen rounding mode.
 // Value as stored on a level: FP32 levels of the bfloat16 storage trial round it.
 template <typename T>

@@ -493,7 +493,6 @@ LevelDev<T> to_dev(const HostLevel& L) {
   d.fxe = L.shape.n - L.per - L.rx;
   d.fye = L.shape.n - L.per - L.ry;
   d.wd = (T)L.wd_fast;
-  for (const int2& e : L.cls) d.maxcnt = std::max(d.maxcnt, (int32_t)e.y);
   for (int k = 0; k < d.nt; ++k) {
     d.c[k] = (T)L.c[k];
     const int dx = L.dxs[k], dy = L.dys[k];
@@ -524,13 +523,14 @@ struct Hier {
   T coarsest_a = T(1);
   int coarsest_zero = 0;  // periodic: the coarsest single node's zero-mean solution is 0
   DenseCoarse<T> dense{};  // m > 0: the coarsest level has m > 1 unknowns (dense solve)
-  // small-level tail (one thread block runs the sub-cycle from tail_level down)
+  // small-level tail (one kernel runs the sub-cycle from tail_level down)
   int tail_level = -1;
   TailDesc<T>* d_tail = nullptr;
   int4* d_prog = nullptr;  // program for a sub-cycle with zero initial guess
   int nops = 0;
+  int nops_cont = 0;       // shared-memory tail: ops of the program that continues from u
+  size_t tail_smem = 0;    // > 0: the tail's levels live in one block's shared memory (bytes)
   int tail_ctas = 1;       // CTAs in the tail's thread-block cluster
-  size_t tail_smem = 0;    // > 0: the tail's levels live in shared memory (bytes)
   std::vector<TileLevel> tiles;  // FP32 levels: TMA tile kernels (tiles.h) where eligible
 };
 
@@ -846,35 +846,72 @@ mg_status upload_dense(mg_handle* h, const std::vector<double>& G, const std::ve
   return MG_OK;
 }
 
+// The class rows as group records (GroupRec), maxg to a class; empty (maxg = 0) if some
+// group has more than kGroupMax terms.
+template <typename T>
+std::vector<GroupRec<T>> group_records(const HostLevel& L, int32_t& maxg) {
+  maxg = 0;
+  for (const int2& e : L.cls) {
+    int32_t g = 0, m = 0;
+    for (int k = e.x; k < e.x + e.y; ++k) {
+      if (L.tstart[k]) ++g, m = 0;
+      if (++m > kGroupMax) {
+        maxg = 0;
+        return {};
+      }
+    }
+    maxg = std::max(maxg, g);
+  }
+  std::vector<GroupRec<T>> out(L.cls.size() * maxg);
+  if (!out.empty()) std::memset(static_cast<void*>(out.data()), 0, out.size() * sizeof(GroupRec<T>));
+  for (size_t c = 0; c < L.cls.size(); ++c) {
+    GroupRec<T>* r = out.data() + c * maxg - 1;
+    for (int k = L.cls[c].x; k < L.cls[c].x + L.cls[c].y; ++k) {
+      if (L.tstart[k]) (++r)->c = (T)L.tc[k];
+      const int dx = L.tdx[k], dy = L.tdy[k];
+      r->d[r->cnt++] = L.shape.kind == kRot ? 4 * dy * L.pitch + 2 * dx + (dy & 1)
+                                            : 4 * (dy * L.pitch + dx) + ((dx + dy) & 1);
+    }
+  }
+  return out;
+}
+
+// The level's descriptor and tables in one allocation, filled by one copy.
 template <typename T>
 mg_status upload_level(mg_handle* h, const HostLevel& L, LevelPair<T>& P, int bf16 = 0) {
   P.h = to_dev<T>(L);
   P.h.bf16 = bf16;
-  int2* cls;
-  T* cwd;
-  ClassTerm<T>* terms;
+  const std::vector<GroupRec<T>> groups = group_records<T>(L, P.h.maxg);
+  size_t bytes = 0;
+  auto place = [&](size_t n) {
+    const size_t at = bytes;
+    bytes += (n + 255) & ~(size_t)255;
+    return at;
+  };
+  const size_t o_dev = place(sizeof(LevelDev<T>)), o_cls = place(L.cls.size() * sizeof(int2)),
+               o_wd = place(L.cls_wd.size() * sizeof(T)), o_terms = place(L.tdx.size() * sizeof(ClassTerm<T>)),
+               o_groups = place(groups.size() * sizeof(GroupRec<T>));
+  char* dev;
   mg_status st;
-  const size_t nt = std::max<size_t>(L.tdx.size(), 1);
-  if ((st = device_alloc(h, (void**)&cls, L.cls.size() * sizeof(int2))) != MG_OK) return st;
-  if ((st = device_alloc(h, (void**)&cwd, L.cls_wd.size() * sizeof(T))) != MG_OK) return st;
-  if ((st = device_alloc(h, (void**)&terms, nt * sizeof(ClassTerm<T>))) != MG_OK) return st;
-  std::vector<T> wd(L.cls_wd.begin(), L.cls_wd.end());
-  std::vector<ClassTerm<T>> tt(L.tdx.size());
-  for (size_t k = 0; k < tt.size(); ++k) {
-    std::memset(&tt[k], 0, sizeof(tt[k]));
+  if ((st = device_alloc(h, (void**)&dev, bytes)) != MG_OK) return st;
+  std::vector<char> blob(bytes, 0);
+  std::memcpy(blob.data() + o_cls, L.cls.data(), L.cls.size() * sizeof(int2));
+  T* wd = reinterpret_cast<T*>(blob.data() + o_wd);
+  for (size_t k = 0; k < L.cls_wd.size(); ++k) wd[k] = (T)L.cls_wd[k];
+  ClassTerm<T>* tt = reinterpret_cast<ClassTerm<T>*>(blob.data() + o_terms);
+  for (size_t k = 0; k < L.tdx.size(); ++k) {
     tt[k].c = (T)L.tc[k];
     tt[k].dx = L.tdx[k] + (L.tstart[k] ? kTermStart : 0);
     tt[k].dy = L.tdy[k];
   }
-  CK(cudaMemcpyAsync(cls, L.cls.data(), L.cls.size() * sizeof(int2), cudaMemcpyHostToDevice, h->priv));
-  CK(cudaMemcpyAsync(cwd, wd.data(), wd.size() * sizeof(T), cudaMemcpyHostToDevice, h->priv));
-  if (!tt.empty())
-    CK(cudaMemcpyAsync(terms, tt.data(), tt.size() * sizeof(ClassTerm<T>), cudaMemcpyHostToDevice, h->priv));
-  P.h.cls = cls;
-  P.h.cls_wd = cwd;
-  P.h.terms = terms;
-  if ((st = device_alloc(h, (void**)&P.d, sizeof(LevelDev<T>))) != MG_OK) return st;
-  CK(cudaMemcpyAsync(P.d, &P.h, sizeof(LevelDev<T>), cudaMemcpyHostToDevice, h->priv));
+  if (!groups.empty()) std::memcpy(blob.data() + o_groups, groups.data(), groups.size() * sizeof(GroupRec<T>));
+  P.d = reinterpret_cast<LevelDev<T>*>(dev + o_dev);
+  P.h.cls = reinterpret_cast<const int2*>(dev + o_cls);
+  P.h.cls_wd = reinterpret_cast<const T*>(dev + o_wd);
+  P.h.terms = reinterpret_cast<const ClassTerm<T>*>(dev + o_terms);
+  P.h.groups = reinterpret_cast<const GroupRec<T>*>(dev + o_groups);
+  std::memcpy(blob.data() + o_dev, &P.h, sizeof(LevelDev<T>));
+  CK(cudaMemcpyAsync(dev, blob.data(), bytes, cudaMemcpyHostToDevice, h->priv));
   return MG_OK;
 }
 
@@ -1071,13 +1108,14 @@ mg_status cycle_level(const Ctx& c, int l, T* U, const T* F, bool zero_init, boo
   const int lmax = (int)h->host.size() - 1;
   mg_status st;
   if (l == H.tail_level) {
-    // the program starts with the zeroing op; skip it to continue from U
-    const int4* prog = zero_init ? H.d_prog : H.d_prog + 1;
-    const int nops = zero_init ? H.nops : H.nops - 1;
     Bracket b(h, l, MG_KERNEL_SMOOTH, c.s);
-    if (H.tail_smem > 0)
-      LAUNCH(h, 1, launch_tail_smem<T>(H.d_tail, H.tail_smem, prog, nops, c.exact, c.s));
-    else LAUNCH(h, 1, launch_tail<T>(H.tail_ctas, H.d_tail, prog, nops, c.exact, c.s));
+    if (H.tail_smem > 0) {  // two programs: from u = 0, then (after it) the one that continues from U
+      LAUNCH(h, 1, launch_tail_smem<T>(H.d_tail, H.tail_smem, zero_init ? H.d_prog : H.d_prog + H.nops,
+                                       zero_init ? H.nops : H.nops_cont, zero_init ? 1 : 0, c.exact, c.s));
+    } else {  // the program starts with the zeroing op; skip it to continue from u
+      const int4* prog = zero_init ? H.d_prog : H.d_prog + 1;
+      LAUNCH(h, 1, launch_tail<T>(H.tail_ctas, H.d_tail, prog, zero_init ? H.nops : H.nops - 1, c.exact, c.s));
+    }
     return MG_OK;
   }
   // FP32 levels with tile kernels: nu1 sweeps from u = 0 in one kernel, the residual
@@ -1268,21 +1306,40 @@ void emit_tail(const mg_handle* h, int l, bool zero, std::vector<int4>& prog, bo
   for (int k = 0; k < h->opt.nu2; ++k) prog.push_back(make_int4(kOpSmooth, l, 0, 0));
 }
 
+// The shared-memory tail's program (launch_tail_smem); `start`: from u = 0. Where the
+// smoother allows it the first half-sweep from 0 is part of the op before (the parent's
+// restriction, or the top level's zeroing op).
+void emit_tail_smem(const mg_handle* h, int l, bool start, std::vector<int4>& prog, bool top) {
+  const int lmax = (int)h->host.size() - 1;
+  const int zs = h->opt.smoother == MG_SMOOTH_REDBLACK && h->opt.nu1 >= 1 ? 1 : 0;
+  if (start && (top || !zs)) prog.push_back(make_int4(kOpZero, l, zs, 0));
+  for (int k = 0; k < h->opt.nu1; ++k) prog.push_back(make_int4(kOpSmooth, l, start && zs && k == 0 ? 1 : 0, 0));
+  prog.push_back(make_int4(kOpResRestrict, l, l + 1 < lmax ? zs : 0, 0));
+  if (l + 1 == lmax) {
+    prog.push_back(make_int4(kOpCoarsest, lmax, 0, 0));
+  } else {
+    for (int g = 0; g < gamma_at(h, l); ++g) emit_tail_smem(h, l + 1, g == 0, prog, false);
+  }
+  prog.push_back(make_int4(kOpProlong, l, 0, 0));
+  for (int k = 0; k < h->opt.nu2; ++k) prog.push_back(make_int4(kOpSmooth, l, 0, 0));
+}
+
 // Hand every level from the first one (below the finest) with at most
 // `max_unknowns` unknowns down to the coarsest to the tail kernel.
 // smem_elems > 0: instead of the unknowns threshold, take the first level (below the
-// finest) from which all levels' u, t, f, d fit in that many shared-memory elements,
+// finest) from which all levels' u, t and f fit in that many shared-memory elements,
 // and run the tail from shared memory.
 template <typename T>
 mg_status build_tail(mg_handle* h, int64_t max_unknowns, int64_t smem_elems = 0) {
   Hier<T>& H = hier<T>(h);
   const int nl = (int)h->host.size();
   int lt = -1;
+  int64_t elems = 0;
   if (smem_elems > 0) {
-    int64_t acc = 0;
     for (int l = nl - 1; l >= 1; --l) {
-      acc += 4 * (int64_t)h->host[l].rows * h->host[l].cols;
-      if (acc > smem_elems) break;
+      const int64_t e = elems + 3 * (int64_t)h->host[l].rows * h->host[l].pitch;
+      if (e > smem_elems) break;
+      elems = e;
       if (l + 1 < nl) lt = l;
     }
   } else {
@@ -1295,22 +1352,18 @@ mg_status build_tail(mg_handle* h, int64_t max_unknowns, int64_t smem_elems = 0)
   if (smem_elems > 0) {
     int off = 0;
     for (int l = lt; l < nl; ++l) {
-      const int e = h->host[l].rows * h->host[l].cols;
+      const int e = h->host[l].rows * h->host[l].pitch;
       td.sm_u[l] = off;
       td.sm_t[l] = off + e;
       td.sm_f[l] = off + 2 * e;
-      td.sm_d[l] = off + 3 * e;
-      off += 4 * e;
+      off += 3 * e;
     }
-    int maxcnt = 1;
-    for (int l = lt; l < nl; ++l) maxcnt = std::max(maxcnt, (int)H.L[l].h.maxcnt);
-    const TailSmemPlan plan = tail_smem_plan<T>(off, maxcnt, H.dense.m);
-    if (plan.octs == 0) return MG_OK;  // no tail
+    const size_t bytes = tail_smem_bytes<T>(off, nl - lt, H.dense.m);
+    if (bytes > kTailSmemMaxBytes) return MG_OK;  // no tail
     td.sm_top = lt;
     td.sm_elems = off;
-    td.sm_octs = plan.octs;
-    td.sm_K = plan.K;
-    H.tail_smem = plan.bytes;
+    td.nlev = nl;
+    H.tail_smem = bytes;
   }
   for (int l = 0; l < nl; ++l) {
     td.L[l] = H.L[l].d;
@@ -1321,44 +1374,48 @@ mg_status build_tail(mg_handle* h, int64_t max_unknowns, int64_t smem_elems = 0)
     td.transfer[l] = l + 1 < nl ? h->transfer[l] : 0;
   }
   td.smoother = h->opt.smoother;
-  td.nlev = nl;
   td.coarsest_idx = H.coarsest_idx;
   td.coarsest_a = H.coarsest_a;
   td.coarsest_zero = H.coarsest_zero;
   td.dense = H.dense;
   std::vector<int4> prog;
-  emit_tail(h, lt, true, prog, true);
+  if (H.tail_smem > 0) {
+    emit_tail_smem(h, lt, true, prog, true);
+    H.nops = (int)prog.size();
+    emit_tail_smem(h, lt, false, prog, true);
+    H.nops_cont = (int)prog.size() - H.nops;
+  } else {
+    emit_tail(h, lt, true, prog, true);
+    H.nops = (int)prog.size();
+  }
   mg_status st;
   if ((st = device_alloc(h, (void**)&H.d_tail, sizeof(td))) != MG_OK) return st;
   if ((st = device_alloc(h, (void**)&H.d_prog, prog.size() * sizeof(int4))) != MG_OK) return st;
   CK(cudaMemcpyAsync(H.d_tail, &td, sizeof(td), cudaMemcpyHostToDevice, h->priv));
   CK(cudaMemcpyAsync(H.d_prog, prog.data(), prog.size() * sizeof(int4), cudaMemcpyHostToDevice, h->priv));
-  H.nops = (int)prog.size();
   H.tail_level = lt;
   H.tail_ctas = tail_ctas<T>(h->opt.fma_contract == 0);
   if (h->opt.tail_ctas > 0) H.tail_ctas = std::min(H.tail_ctas, (int)h->opt.tail_ctas);
   return MG_OK;
 }
 
-// Largest level (unknowns) run by the tail cluster (16 SMs). With the cycle in a
-// CUDA graph a small level's full-grid launch costs little, and the tail's per-phase
-// latency on 16 SMs only wins for the last few levels (measured on GB300).
-constexpr int64_t kTailUnknownsFp64 = 256;
-// FP32 inner hierarchies by default keep their small levels in one block's shared
-// memory (up to 6K elements = 24 KB for u, t, f and d of every tail level). Measured on
-// GB300, mixed solves (order 4, N(0,1) right-hand side; budget 4K / 6K / 8K / 12K / 16K /
-// 24K elements): 257^2 n_min 16 to 1e-8 1.75 / 1.75 / 1.78 / 1.78 / 1.95 / 1.94 ms;
-// 257^2 n_min 2 2.27 / 2.15 / 2.16 / 2.20 / 2.20 / 2.39; 2049^2 n_min 16 4.97-5.03 at 4K-12K,
-// 5.15-5.16 above; 4097^2 n_min 16 to 1e-10 11.38-11.43 at 4K-12K, 11.64-11.65 above.
-// A larger tail runs more levels on one SM, and their boundary-class term records no
-// longer fit the L1 left beside the shared memory; no tail at all is slower still
-// (257^2 n_min 2: 2.71 ms).
-constexpr int64_t kTailSmemElemsFp32 = 6 * 1024;
-// FP64 hierarchies by default use a shared-memory tail too, of 3K elements (24 KB);
-// measured on GB300 (FP64 solve, 4097^2 / 513^2 / 129^2): cluster tail 65.8 / 8.45 /
-// 5.55 ms, 3K 65.0 / 7.64 / 4.77, 6K 65.4 / 8.10 / 5.25, 12K 66.6 / 9.42 / 6.33.
-// tail_unknowns > 0 selects the cluster tail with that threshold.
-constexpr int64_t kTailSmemElemsFp64 = 3 * 1024;
+// The tail that the options ask for. V and Wn cycles by default have none: small levels as
+// separate launches with programmatic dependent launch are the fastest form (measured on
+// GB300, launches / their sub-cycle in one block's shared memory, best of five budgets:
+// FP64 128^2 1.88 / 1.94 ms, FP64 4096^2 38.4 / 38.6, mixed 4096^2 9.63 / 9.76; in a cluster
+// of 16 CTAs slower still, as a cluster barrier after stores into the other CTAs' shared
+// memory takes 0.65-1.5 us and an empty kernel in a graph 0.85 us). A W cycle visits level
+// l 2^l times, so there every level kept out of the launch list halves its length.
+// Budgets in values of u, t and f; three W cycles of 256^2, order 4: mixed 415 / 403 ms with
+// 3K / 6K, FP64 782 ms with 3K and 4.5K and 9-13% more with 7K and 13.5K.
+constexpr int64_t kTailSmemElemsFp32 = 6 * 1024, kTailSmemElemsFp64 = 4608;
+template <typename T>
+mg_status default_tail(mg_handle* h) {
+  const mg_options& o = h->opt;
+  if (o.tail_unknowns > 0) return build_tail<T>(h, o.tail_unknowns);
+  if (o.tail_unknowns < 0 || o.gamma != 2) return MG_OK;
+  return build_tail<T>(h, 0, sizeof(T) == 8 ? kTailSmemElemsFp64 : kTailSmemElemsFp32);
+}
 
 // Power of two near 1 / rms of a residual with squared norm r2 over m unknowns, so
 // that the FP32 copy of the residual stays far from underflow and overflow.
@@ -1522,21 +1579,14 @@ mg_status mg_setup(const mg_grid* grid, int order, mg_coarsening coarsening, mg_
   h->h64.coarsest_a = ca;
   h->h64.coarsest_zero = C.per;
   if (!cij.empty() && (st = upload_dense<double>(h, cG, cij, h->h64.dense)) != MG_OK) return fail(st);
-  auto tail_limit = [&](int64_t dflt) -> int64_t {
-    return o.tail_unknowns < 0 ? 0 : (o.tail_unknowns > 0 ? (int64_t)o.tail_unknowns : dflt);
-  };
-  if (o.tail_unknowns == 0 && kTailSmemElemsFp64 > 0) st = build_tail<double>(h, 0, kTailSmemElemsFp64);
-  else st = build_tail<double>(h, tail_limit(kTailUnknownsFp64));
-  if (st != MG_OK) return fail(st);
+  if ((st = default_tail<double>(h)) != MG_OK) return fail(st);
   if (o.precision == MG_PREC_MIXED_FP32) {
     if ((st = alloc_hier<float>(h, false)) != MG_OK) return fail(st);
     h->h32.coarsest_idx = cidx;
     h->h32.coarsest_a = (float)ca;
     h->h32.coarsest_zero = C.per;
     if (!cij.empty() && (st = upload_dense<float>(h, cG, cij, h->h32.dense)) != MG_OK) return fail(st);
-    if (o.tail_unknowns == 0) st = build_tail<float>(h, 0, kTailSmemElemsFp32);
-    else st = build_tail<float>(h, tail_limit(0));
-    if (st != MG_OK) return fail(st);
+    if ((st = default_tail<float>(h)) != MG_OK) return fail(st);
     // TMA tile kernels on the large eligible FP32 levels above the tail (sweep_kernel 0)
     h->h32.tiles.assign(nl, TileLevel());
     if (o.sweep_kernel == 0 && o.smoother == MG_SMOOTH_REDBLACK)

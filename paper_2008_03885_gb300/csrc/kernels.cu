@@ -28,23 +28,23 @@ struct SweepArgs {
   LevelGeo<T> L;
   const LevelDev<T>* Lp;
   StripGeo S;
-  int32_t colour, sblocks, gx, K;
+  int32_t colour, sblocks, gx;
 };
 
-// Terms a lane of an octet fetches at once: rows of the 5/9-point levels have at most 9
-// terms, the wide Galerkin rows up to 45 (longer ones take several batches).
-constexpr int kStripBatchNt = 2, kStripBatchGen = 6;
+// Group records a lane of an octet fetches at once: boundary rows of the 5/9-point levels
+// have at most 6 groups, those of the 45-point Galerkin levels up to 15 (rows with more
+// take several batches).
+constexpr int kRecsNt = 1, kRecsGen = 2;
 
 template <typename T, bool EXACT, int NT, bool PER>
 __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value)
-    k_half_sweep_nt(const __grid_constant__ SweepArgs<T> A, const T* __restrict__ uin, const T* __restrict__ f,
-                    T* __restrict__ uout) {
-  extern __shared__ __align__(16) unsigned char strip_smem[];
+    k_half_sweep_nt(const __grid_constant__ SweepArgs<T> A, const T* uin, const T* f, T* __restrict__ uout) {
   constexpr int kRows = RowsPer<T>::value;
   const LevelGeo<T>& L = A.L;
   const int red = A.colour;
+  pdl_trigger();
   if ((int)blockIdx.x < A.sblocks) {
-    strip_rows<T, EXACT, kStripBatchNt, kRowRelax>(L, A.S, red, blockIdx.x, uin, f, uout, strip_smem, A.K);
+    strip_rows<T, EXACT, kRecsNt, kRowRelax>(L, A.S, red, blockIdx.x, uin, f, uout);
     return;
   }
   const int by = ((int)blockIdx.x - A.sblocks) / A.gx, bx = (int)blockIdx.x - A.sblocks - by * A.gx;
@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value)
     d0[k] = A.Lp->delta[0][k];
     d1[k] = A.Lp->delta[1][k];
   }
+  pdl_wait();
   const T wd = L.wd;
   const int n = L.n;
   constexpr int lo = PER ? 0 : 1;
@@ -112,13 +113,12 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value)
 
 template <typename T, bool EXACT, int NT, bool PER>
 __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value)
-    k_residual_nt(const __grid_constant__ SweepArgs<T> A, const T* __restrict__ u, const T* __restrict__ f,
-                  T* __restrict__ d) {
-  extern __shared__ __align__(16) unsigned char strip_smem[];
+    k_residual_nt(const __grid_constant__ SweepArgs<T> A, const T* u, const T* f, T* __restrict__ d) {
   constexpr int kRows = RowsPer<T>::value;
   const LevelGeo<T>& L = A.L;
+  pdl_trigger();
   if ((int)blockIdx.x < A.sblocks) {
-    strip_rows<T, EXACT, kStripBatchNt, kRowResidual>(L, A.S, kAllNodes, blockIdx.x, u, f, d, strip_smem, A.K);
+    strip_rows<T, EXACT, kRecsNt, kRowResidual>(L, A.S, kAllNodes, blockIdx.x, u, f, d);
     return;
   }
   const int by = ((int)blockIdx.x - A.sblocks) / A.gx, bx = (int)blockIdx.x - A.sblocks - by * A.gx;
@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value)
     d0[k] = A.Lp->delta[0][k];
     d1[k] = A.Lp->delta[1][k];
   }
+  pdl_wait();
   const int q = bx * kBX + threadIdx.x;
   if (q >= L.cols) return;
   const int jb = by * (kBY * kRows) + threadIdx.y;
@@ -207,18 +208,18 @@ constexpr int kGenDeepRows = 2048;
 
 template <typename T, bool EXACT, bool DEEP>
 __global__ void __launch_bounds__(kBX * kBY, GenCfg<T, DEEP>::min_blocks)
-    k_half_sweep_gen(const __grid_constant__ SweepArgs<T> A, const T* __restrict__ uin, const T* __restrict__ f,
-                     T* __restrict__ uout) {
-  extern __shared__ __align__(16) unsigned char strip_smem[];
+    k_half_sweep_gen(const __grid_constant__ SweepArgs<T> A, const T* uin, const T* f, T* __restrict__ uout) {
   const LevelGeo<T>& L = A.L;
   const int red = A.colour;
+  pdl_trigger();
   if ((int)blockIdx.x < A.sblocks) {
-    strip_rows<T, EXACT, kStripBatchGen, kRowRelax>(L, A.S, red, blockIdx.x, uin, f, uout, strip_smem, A.K);
+    strip_rows<T, EXACT, kRecsGen, kRowRelax>(L, A.S, red, blockIdx.x, uin, f, uout);
     return;
   }
   const int by = ((int)blockIdx.x - A.sblocks) / A.gx, bx = (int)blockIdx.x - A.sblocks - by * A.gx;
   __shared__ StencilSmem<T> sm;
   if (!A.S.all) stage_stencil(*A.Lp, sm);
+  pdl_wait();
   int i, j = by * blockDim.y + threadIdx.y;
   if (j < L.lo || j >= L.n) return;
   if (L.kind == kAxis) {
@@ -248,17 +249,17 @@ __global__ void __launch_bounds__(kBX * kBY, GenCfg<T, DEEP>::min_blocks)
 
 template <typename T, bool EXACT, bool DEEP>
 __global__ void __launch_bounds__(kBX * kBY, GenCfg<T, DEEP>::min_blocks)
-    k_residual_gen(const __grid_constant__ SweepArgs<T> A, const T* __restrict__ u, const T* __restrict__ f,
-                   T* __restrict__ d) {
-  extern __shared__ __align__(16) unsigned char strip_smem[];
+    k_residual_gen(const __grid_constant__ SweepArgs<T> A, const T* u, const T* f, T* __restrict__ d) {
   const LevelGeo<T>& L = A.L;
+  pdl_trigger();
   if ((int)blockIdx.x < A.sblocks) {
-    strip_rows<T, EXACT, kStripBatchGen, kRowResidual>(L, A.S, kAllNodes, blockIdx.x, u, f, d, strip_smem, A.K);
+    strip_rows<T, EXACT, kRecsGen, kRowResidual>(L, A.S, kAllNodes, blockIdx.x, u, f, d);
     return;
   }
   const int by = ((int)blockIdx.x - A.sblocks) / A.gx, bx = (int)blockIdx.x - A.sblocks - by * A.gx;
   __shared__ StencilSmem<T> sm;
   stage_stencil(*A.Lp, sm);
+  pdl_wait();
   const int q = bx * kBX + threadIdx.x, j = by * blockDim.y + threadIdx.y;
   const int i = L.kind == kRot ? 2 * q + (j & 1) : q;
   if (!fast_node(L, i, j)) return;
@@ -448,19 +449,9 @@ __host__ __device__ constexpr double rt_w(int tr, int k) {
   return tr == kStandard ? (rt_dx(tr, k) == 0 ? 2 : 1) * (rt_dy(tr, k) == 0 ? 2 : 1) * 0.0625 : (k == 2 ? 0.5 : 0.125);
 }
 
-// Storage position of lattice node (i, j): in the level's global storage, or in the
-// compact rows x cols layout of the shared-memory tail.
-template <typename T>
-__device__ __forceinline__ int smem_idx(const LevelGeo<T>& L, int i, int j) {
-  return j * L.cols + (L.kind == kRot ? (i >> 1) : i);
-}
 struct GlobalIdx {
   template <typename T>
   __device__ __forceinline__ int64_t operator()(const LevelGeo<T>& L, int i, int j) const { return sidx(L, i, j); }
-};
-struct SmemIdx {
-  template <typename T>
-  __device__ __forceinline__ int64_t operator()(const LevelGeo<T>& L, int i, int j) const { return smem_idx(L, i, j); }
 };
 
 // Periodic transfers: terms (lattice i, j, weight) on level L wrap modulo L.n, are
@@ -805,23 +796,25 @@ __device__ __forceinline__ void store_restricted(const LevelGeo<T>& Lc, T* __res
 
 template <typename T, bool EXACT, bool PER>
 __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value)
-    k_restrict_cubic(const LevelDev<T>* __restrict__ Lfp, const LevelDev<T>* __restrict__ Lcp, const T* __restrict__ d,
-                     T* __restrict__ fc, T* __restrict__ tc) {
-  const LevelDev<T>& Lc = *Lcp;
+    k_restrict_cubic(const __grid_constant__ LevelGeo<T> Lf, const __grid_constant__ LevelGeo<T> Lc,
+                     const T* d, T* __restrict__ fc, T* __restrict__ tc) {
+  pdl_trigger();
+  pdl_wait();
   int i, j;
   if (!thread_node(Lc, i, j) || !interior(Lc, i, j)) return;
-  store_restricted(Lc, fc, tc, i, j, rnd(Lc, restrict_cubic_value<T, EXACT, PER>(*Lfp, d, i, j)));
+  store_restricted(Lc, fc, tc, i, j, rnd(Lc, restrict_cubic_value<T, EXACT, PER>(Lf, d, i, j)));
 }
 
 template <typename T, bool EXACT, bool PER>
 __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value)
-    k_prolong_cubic(const LevelDev<T>* __restrict__ Lfp, const LevelDev<T>* __restrict__ Lcp, const T* uin, T* uf,
-                    const T* __restrict__ vc) {
-  const LevelDev<T>& Lf = *Lfp;
+    k_prolong_cubic(const __grid_constant__ LevelGeo<T> Lf, const __grid_constant__ LevelGeo<T> Lc, const T* uin, T* uf,
+                    const T* vc) {
+  pdl_trigger();
+  pdl_wait();
   int i, j;
   if (!thread_node(Lf, i, j) || !interior(Lf, i, j)) return;
   const int64_t at = sidx(Lf, i, j);
-  uf[at] = rnd(Lf, Arith<T>::add(uin[at], prolong_cubic_value<T, EXACT, PER>(*Lcp, vc, i, j)));
+  uf[at] = rnd(Lf, Arith<T>::add(uin[at], prolong_cubic_value<T, EXACT, PER>(Lc, vc, i, j)));
 }
 
 // On large levels the restriction and interpolation kernels give each thread
@@ -836,10 +829,10 @@ constexpr int kTransferRows = 4;
 constexpr int kTransferRowsMinLevelRows = 2048;
 
 template <typename T, bool EXACT, bool PER, int ROWS>
-__global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_restrict(const LevelDev<T>* __restrict__ Lfp, const LevelDev<T>* __restrict__ Lcp,
-                           int transfer, const T* __restrict__ d, T* __restrict__ fc, T* __restrict__ tc) {
-  const LevelDev<T>& Lf = *Lfp;
-  const LevelDev<T>& Lc = *Lcp;
+__global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_restrict(const __grid_constant__ LevelGeo<T> Lf, const __grid_constant__ LevelGeo<T> Lc,
+                           int transfer, const T* d, T* __restrict__ fc, T* __restrict__ tc) {
+  pdl_trigger();
+  pdl_wait();
   const int q = blockIdx.x * kBX + threadIdx.x;
   if (q >= Lc.cols) return;
   const int jb = blockIdx.y * (kBY * ROWS) + threadIdx.y;
@@ -866,10 +859,10 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_restrict(con
 // PAIR: an axis fine level, one thread per node pair (2p, 2p + 1); otherwise one thread
 // per storage column (rotated fine levels hold one interpolation kind per row).
 template <typename T, bool EXACT, bool PER, int ROWS, bool PAIR>
-__global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_prolong_add(const LevelDev<T>* __restrict__ Lfp, const LevelDev<T>* __restrict__ Lcp,
-                              int transfer, const T* uin, T* uf, const T* __restrict__ vc) {
-  const LevelDev<T>& Lf = *Lfp;
-  const LevelDev<T>& Lc = *Lcp;
+__global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_prolong_add(const __grid_constant__ LevelGeo<T> Lf, const __grid_constant__ LevelGeo<T> Lc,
+                              int transfer, const T* uin, T* uf, const T* vc) {
+  pdl_trigger();
+  pdl_wait();
   const bool axis = Lf.kind == kAxis;
   const int t = blockIdx.x * kBX + threadIdx.x;
   const int i0 = PAIR ? 2 * t : 0;
@@ -900,7 +893,9 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<T>::value) k_prolong_add(
 // Exact solve on the one-unknown coarsest level: u = f / a_pp (Dirichlet), or the
 // zero-mean solution u = 0 of a periodic single node, whose operator row is zero.
 template <typename T>
-__global__ void k_coarsest(int64_t idx, T a, int zero_mean, const T* __restrict__ f, T* __restrict__ u) {
+__global__ void k_coarsest(int64_t idx, T a, int zero_mean, const T* f, T* __restrict__ u) {
+  pdl_trigger();
+  pdl_wait();
   if (threadIdx.x == 0 && blockIdx.x == 0) u[idx] = zero_mean ? T(0) : Arith<T>::div(f[idx], a);
 }
 
@@ -1015,8 +1010,10 @@ __device__ __forceinline__ void dense_coarse_vec(const DenseCoarse<T>& C, const 
 
 template <typename T, bool EXACT>
 __global__ void __launch_bounds__(1024) k_coarsest_dense(DenseCoarse<T> C, const __grid_constant__ LevelGeo<T> L,
-                                                         const T* __restrict__ f, T* __restrict__ u) {
+                                                         const T* f, T* __restrict__ u) {
   __shared__ T v[2 * kMaxDense];
+  pdl_trigger();
+  pdl_wait();
   dense_coarse_vec<T, EXACT>(C, L, f, v, u, GlobalIdx(), (int)threadIdx.x, (int)blockDim.x);
 }
 
@@ -1072,9 +1069,10 @@ __global__ void k_resnorm_partial(const LevelDev<T>* __restrict__ Lp, const T* _
 // without the stencil gathers (and replaces zeroing u, since the black half-sweep that
 // follows writes every unknown of u).
 template <typename T>
-__global__ void k_first_half_zero(const LevelDev<T>* __restrict__ Lp, const T* __restrict__ f, T* __restrict__ t,
+__global__ void k_first_half_zero(const __grid_constant__ LevelGeo<T> L, const T* f, T* __restrict__ t,
                                   int red) {
-  const LevelDev<T>& L = *Lp;
+  pdl_trigger();
+  pdl_wait();
   int i, j;
   if (!thread_node(L, i, j) || !interior(L, i, j)) return;
   const int64_t at = sidx(L, i, j);
@@ -1518,169 +1516,236 @@ __global__ void __launch_bounds__(kBX * kBY)
 }
 
 // ---- shared-memory-resident tail ---------------------------------------------
-// Levels from sm_top down live in one block's shared memory in a compact rows x cols
-// layout; node (i, j) of a level is at j * cols + (rot ? i >> 1 : i). Operator rows are
-// evaluated by octets of lanes (rows.cuh), sm_octs of them, from class rows that stay in
-// L1 after their first use. Arithmetic per node is the same as relax_value / apply_at /
-// restrict_value / prolong_value.
+// The levels from sm_top down live in one block's shared memory, each in its storage
+// layout, and the block runs their whole sub-cycle with a barrier between phases. Class
+// rows are evaluated by octets of lanes in FP64 and by one thread a node in FP32 (rows.cuh;
+// with the values in shared memory and the records in L1 the octets' chain of shuffles is
+// the longer one); arithmetic per node is the same as relax_value / apply_at /
+// restrict_value / prolong_value. Measured, three W cycles of 256^2, order 4: FP64 1197 ->
+// 782 ms, mixed 485 -> 403 ms (548 with octets) against one thread per storage element.
 //
 // A sweep reads the level's current array A and writes the other one, B: the red phase
 // reads A and writes B's red nodes, the black phase reads B at red and A at black nodes
 // and writes B's black nodes; then the arrays change roles (bit l of `flip`: level l's
-// current array is t). No colour is copied.
+// current array is t). No colour is copied. The residual goes to B as well.
+//
 // 512 threads (64 octets, 128 registers): with 1024 the row evaluation spilled in FP64.
+//
+// Fast nodes of a level with more than kTailThreadNodes nodes to update are evaluated by
+// one thread each from the level's interior stencil (staged in shared memory, uniform over
+// a warp): a lone octet is the shorter chain, but past about two octet warps to each FP64
+// unit (FP32: issue slots) the threads' 60 FP64 instructions for 32 nodes beat 20 for four.
 constexpr int kTailSmemThreads = 512;
 template <typename T>
-struct TailSmem {
-  static __host__ __device__ __forceinline__ size_t stage(int sm_elems) {  // byte offset of the octets' staging
-    return ((size_t)sm_elems * sizeof(T) + 15) & ~(size_t)15;
-  }
-};
+constexpr int kTailThreadNodes = sizeof(T) == 8 ? 32 : 16;
+constexpr int kTailStencil = 48;  // longest interior stencil evaluated by threads (others: octets)
 
-// All unknowns of one colour (or all) of a level, one slot each (as make_strips with
-// `all`): slots, and slot -> node.
 template <typename T>
-struct LevelSlots {
-  int lo, hi, rstep, cstep, first, w, total, colour, kind;
-  __device__ __forceinline__ LevelSlots(const LevelGeo<T>& L, int c) : lo(L.lo), hi(L.n - 1), colour(c), kind(L.kind) {
-    rstep = (kind == kRot && c != kAllNodes) ? 2 : 1;
-    cstep = (kind == kAxis && c == kAllNodes) ? 1 : 2;
-    first = rstep == 2 ? lo + ((lo ^ c) & 1) : lo;
-    w = (hi - lo) / cstep + 1;
-    total = (first > hi ? 0 : (hi - first) / rstep + 1) * w;
-  }
-  __device__ __forceinline__ bool node(int slot, int& i, int& j) const {
-    if (slot >= total) return false;
-    const int r = slot / w, s = slot - r * w;
-    j = first + r * rstep;
-    if (cstep == 1) {
-      i = lo + s;
-    } else {
-      const int par = kind == kRot ? (j & 1) : ((j ^ colour) & 1);
-      i = lo + ((lo ^ par) & 1) + 2 * s;
-    }
-    return i <= hi;
-  }
+__host__ __device__ __forceinline__ size_t tail_stencils(int sm_elems) {  // byte offset of the interior stencils
+  return ((size_t)sm_elems * sizeof(T) + 15) & ~(size_t)15;
+}
+template <typename T>
+__host__ __device__ __forceinline__ size_t tail_scratch(int sm_elems, int nst) {  // and of the dense solve's vectors
+  return tail_stencils<T>(sm_elems) + (size_t)nst * kTailStencil * (sizeof(T) + 2 * sizeof(int));
+}
+
+// Work of a phase over the nodes of one colour (or all) of a level: class nodes S, and the
+// slots of the fast rectangle that threads take (w to a row, rstep rows apart from row
+// `first` on; none: total = 0). Worked out once per launch, not once per phase.
+struct TailPhase {
+  StripGeo S;
+  int32_t first, w, total;
+  uint32_t m;  // slot / w = slot m >> 32 (w = 1: m = 0)
 };
 
+template <typename T>
+__device__ __forceinline__ TailPhase tail_phase(const LevelGeo<T>& L, int c) {
+  TailPhase P;
+  const int rot = L.kind == kRot;
+  const int nodes = (L.n - L.lo) * (L.n - L.lo) / ((rot ? 2 : 1) * (c == kAllNodes ? 1 : 2));
+  P.S = make_strips(L, c, nodes <= kTailThreadNodes<T> || L.nt > kTailStencil);
+  P.first = P.S.rstep == 2 ? L.ry + ((L.ry ^ c) & 1) : L.ry;
+  P.w = P.S.all ? 0 : (L.fxe - L.rx) / P.S.cstep + 1;
+  P.total = P.S.all || P.first > L.fye ? 0 : ((L.fye - P.first) / P.S.rstep + 1) * P.w;
+  P.m = P.w > 1 ? 0xffffffffu / P.w + 1 : 0;
+  return P;
+}
+
+// zero: the sub-cycle starts from u = 0 (the program then starts with kOpZero); otherwise
+// the top level's u is read from global memory.
 template <typename T, bool EXACT>
 __global__ void __launch_bounds__(kTailSmemThreads, 1)
-    k_tail_smem(const TailDesc<T>* __restrict__ D, const int4* __restrict__ prog, int nops) {
+    k_tail_smem(const TailDesc<T>* __restrict__ D, const int4* __restrict__ prog, int nops, int zero) {
   extern __shared__ __align__(16) unsigned char tail_smem[];
   __shared__ LevelGeo<T> geo[kTailMaxLevels];
+  __shared__ uint64_t gst[kTailMaxLevels];
+  __shared__ TailPhase phase[kTailMaxLevels][3];
   T* sm = reinterpret_cast<T*>(tail_smem);
-  const int tid = threadIdx.x, lane = tid & 31, oct = tid >> 3;
-  const int top = D->sm_top, nocts = D->sm_octs, K = D->sm_K;
-  unsigned char* stage = tail_smem + TailSmem<T>::stage(D->sm_elems) + oct * oct_bytes<T>(K);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int top = D->sm_top, nst = D->nlev - top;
   for (int k = tid; k < D->sm_elems; k += kTailSmemThreads) sm[k] = T(0);
   for (int l = top + tid; l < D->nlev; l += kTailSmemThreads) geo[l] = *D->L[l];
+  // interior stencils: coefficients, and per parity of i the storage offset with the term's
+  // colour (0: the node's own) in the lowest bit; group starts as a bit mask
+  T* stc = reinterpret_cast<T*>(tail_smem + tail_stencils<T>(D->sm_elems));
+  int* sto = reinterpret_cast<int*>(stc + nst * kTailStencil);
+  for (int x = tid; x < nst * kTailStencil; x += kTailSmemThreads) {
+    const int l = x / kTailStencil, k = x - l * kTailStencil;
+    const LevelDev<T>& L = *D->L[top + l];
+    if (k == 0) gst[top + l] = (uint64_t)L.gmask[1] << 32 | L.gmask[0];
+    if (k >= L.nt) continue;
+    stc[x] = L.c[k];
+    for (int par = 0; par < 2; ++par) {
+      // colour of the term: parity of dx + dy on axis levels, of the row on rotated ones
+      const int other = (L.kind == kRot ? L.sdy[k] : L.sdx[0][k] + L.sdy[k]) & 1;
+      sto[(2 * l + par) * kTailStencil + k] = L.delta[par][k] * 2 + other;
+    }
+  }
   __syncthreads();
-  {  // top level: u and f from global memory
+  for (int x = tid; x < 3 * nst; x += kTailSmemThreads) phase[top + x / 3][x % 3] = tail_phase(geo[top + x / 3], x % 3);
+  {  // top level: f, and u unless it is zero, from global memory
     const LevelGeo<T>& L = geo[top];
-    for (int k = tid; k < L.rows * L.cols; k += kTailSmemThreads) {
-      const int j = k / L.cols, q = k - j * L.cols;
-      sm[D->sm_u[top] + k] = D->u[top][(int64_t)j * L.pitch + q];
-      sm[D->sm_f[top] + k] = D->f[top][(int64_t)j * L.pitch + q];
+    for (int k = tid; k < L.rows * L.pitch; k += kTailSmemThreads) {
+      if (!zero) sm[D->sm_u[top] + k] = D->u[top][k];
+      sm[D->sm_f[top] + k] = D->f[top][k];
     }
   }
   __syncthreads();
   uint64_t flip = 0;
   auto cur = [&](int l) { return ((flip >> l) & 1) ? D->sm_t[l] : D->sm_u[l]; };
   auto oth = [&](int l) { return ((flip >> l) & 1) ? D->sm_u[l] : D->sm_t[l]; };
-  // fin(k, i, j, (L u)(i, j), cl) in the first lane of the octet of every node of colour
-  // c; a term at a red node reads the array at offset `ra`, at a black one `ba`
-  auto rows = [&](int l, int c, int ra, int ba, auto fin) {
+  // Every node of colour c: its relaxed value (or residual, res) goes to offset out + k. A
+  // term at a red node reads the array at offset ra, at a black one ba. Chunks of work (four
+  // octet nodes, or 32 fast nodes) go round the block's warps.
+  auto rows = [&](int l, int c, int ra, int ba, int out, bool res) {
     const LevelGeo<T>& L = geo[l];
-    const LevelSlots<T> S(L, c);
-    const int cols = L.cols, rot = L.kind == kRot;
-    auto pos = [=](int i, int j) {
-      const int red = rot ? (i & 1) : ((i + j) & 1);
-      return (red ? ra : ba) + j * cols + (rot ? (i >> 1) : i);
+    const T *F = sm + D->sm_f[l], *A = sm + ba;  // a node's own value is in A at either colour
+    const int rot = L.kind == kRot;
+    const TailPhase& P = phase[l][c];
+    const StripGeo& S = P.S;
+    constexpr int kPer = sizeof(T) == 8 ? 4 : 32;  // class nodes to a chunk
+    const int oc = (S.total + kPer - 1) / kPer, chunks = oc + (P.total + 31) / 32;
+    auto val = [&](int k, T v, T wd) {
+      const T r = Arith<T>::sub(F[k], v);
+      if (res) return r;
+      return EXACT ? Arith<T>::add(A[k], Arith<T>::mul(r, wd)) : Arith<T>::fma(r, wd, A[k]);
     };
-    for (int s0 = 0; s0 < S.total; s0 += nocts) {
-      if (oct >= nocts || s0 + (oct & ~3) >= S.total) break;  // uniform over a warp
+    for (int q = tid >> 5; q < chunks; q += kTailSmemThreads / 32) {
       int i = 0, j = 0;
-      const bool on = S.node(s0 + oct, i, j);
-      const int cl = on ? class_of(L, i, j) : 0;
-      const T v = octet_row<T, EXACT, 6>(L, sm, on, i, j, cl, stage, K, pos);
-      if (on && (lane & 7) == 0) fin(smem_idx(L, i, j), v, cl);
+      if (q < oc) {
+        const bool on = strip_node(L, S, c, kPer * q + lane * kPer / 32, i, j);
+        const int cl = on ? class_of(L, i, j) : 0;
+        const T wd = on ? L.cls_wd[cl] : T(0);
+        const int k = (int)sidx(L, i, j), red = is_red(L, i, j);
+        const T *own = sm + k + (red ? ra : ba), *opp = sm + k + (red ? ba : ra);
+        if constexpr (kPer == 32) {
+          if (on) sm[out + k] = val(k, serial_row<T, EXACT>(L, own, opp, i, j, cl), wd);
+        } else {
+          const T v = octet_row<T, EXACT, 2>(L, own, opp, on, i, j, cl, []() {});
+          if (on && (lane & 7) == 0) sm[out + k] = val(k, v, wd);
+        }
+      } else {
+        const int slot = 32 * (q - oc) + lane, r = P.m ? (int)__umulhi((uint32_t)slot, P.m) : slot;
+        j = P.first + r * S.rstep;
+        i = L.rx + (slot - r * P.w) * S.cstep;
+        if (S.cstep == 2) i += (L.rx ^ (rot ? j : j ^ c)) & 1;
+        if (slot >= P.total || i > L.fxe) continue;
+        const int k = (int)sidx(L, i, j), red = is_red(L, i, j);
+        const T *own = sm + k + (red ? ra : ba), *opp = sm + k + (red ? ba : ra);
+        const T* cs = stc + (l - top) * kTailStencil;
+        const int* os = sto + (2 * (l - top) + (rot ? (i & 1) : 0)) * kTailStencil;
+        const uint64_t gs = gst[l];
+        RowSum<T, EXACT> acc;
+        constexpr int U = 8;
+        int t = 0;
+        for (; t + U <= L.nt; t += U) {
+          T x[U];
+#pragma unroll
+          for (int r = 0; r < U; ++r) {
+            const int o = os[t + r];
+            x[r] = (o & 1 ? opp : own)[o >> 1];
+          }
+#pragma unroll
+          for (int r = 0; r < U; ++r) acc.add(cs[t + r], x[r], (gs >> (t + r)) & 1);
+        }
+        for (; t < L.nt; ++t) {
+          const int o = os[t];
+          acc.add(cs[t], (o & 1 ? opp : own)[o >> 1], (gs >> t) & 1);
+        }
+        sm[out + k] = val(k, acc.value(), L.wd);
+      }
     }
   };
+  // The first half-sweep from u = 0 at element k with right-hand side v: B's red node
+  // relaxed, A's black node 0 (A may hold an earlier visit's values).
+  auto start_at = [&](int l, int k, int i, int j, T v) {
+    const LevelGeo<T>& L = geo[l];
+    if (is_red(L, i, j)) sm[oth(l) + k] = relax_from_zero(v, node_wd(L, i, j));
+    else sm[cur(l) + k] = T(0);
+  };
+  // body(k, i, j) at every unknown of a level, a warp to a row
+  auto each = [&](const LevelGeo<T>& L, auto body) {
+    for (int j = L.lo + (tid >> 5); j < L.n; j += kTailSmemThreads / 32)
+      for (int q = lane; q < L.cols; q += 32) {
+        const int i = L.kind == kRot ? 2 * q + (j & 1) : q;
+        if (i >= L.lo && i < L.n) body(j * L.pitch + q, i, j);
+      }
+  };
+  int4 next = prog[0];
   for (int p = 0; p < nops; ++p) {
-    const int4 op = prog[p];
+    const int4 op = next;
+    if (p + 1 < nops) next = prog[p + 1];
     const int l = op.y;
     const LevelGeo<T>& L = geo[l];
-    const int total = L.rows * L.cols;
     const T* F = sm + D->sm_f[l];
-    int i, j;
-    if (op.x == kOpZero) {
-      T* U = sm + cur(l);
-      for (int k = tid; k < total; k += kTailSmemThreads) U[k] = T(0);
-    } else if (op.x == kOpSmooth) {
+    if (op.x == kOpZero) {  // z: with the first half-sweep from 0
+      each(L, [&](int k, int i, int j) {
+        if (op.z) start_at(l, k, i, j, F[k]);
+        else sm[cur(l) + k] = T(0);
+      });
+    } else if (op.x == kOpSmooth || op.x == kOpResRestrict) {
+      const bool res = op.x == kOpResRestrict;
       const int ca = cur(l), cb = oth(l);
-      auto relax = [&](int k, T v, int cl) {
-        const T r = Arith<T>::sub(F[k], v), wd = L.cls_wd[cl];
-        const T x = sm[ca + k];
-        sm[cb + k] = EXACT ? Arith<T>::add(x, Arith<T>::mul(r, wd)) : Arith<T>::fma(r, wd, x);
-      };
-      if (D->smoother == 0) {
-        if (op.z) {  // first half-sweep from u = 0 (op.z: the array was not zeroed)
-          for (int k = tid; k < total; k += kTailSmemThreads) {
-            if (!tail_node(L, k, i, j)) continue;
-            if (is_red(L, i, j)) sm[cb + k] = relax_from_zero(F[k], node_wd(L, i, j));
-            else sm[ca + k] = T(0);
-          }
-        } else {
-          rows(l, kRedNodes, ca, ca, relax);
-        }
+      // kOpSmooth with z: the red half-sweep is done
+      int c = res || D->smoother != 0 ? kAllNodes : op.z ? kBlackNodes : kRedNodes;
+      for (;;) {
+        rows(l, c, c == kBlackNodes ? cb : ca, ca, cb, res);
+        if (c != kRedNodes) break;
         __syncthreads();
-        rows(l, kBlackNodes, cb, ca, relax);
-      } else {
-        rows(l, kAllNodes, ca, ca, relax);
+        c = kBlackNodes;
       }
-      flip ^= 1ull << l;
-    } else if (op.x == kOpResRestrict) {
-      T* Dd = sm + D->sm_d[l];
-      const int c = cur(l);
-      rows(l, kAllNodes, c, c, [&](int k, T v, int) { Dd[k] = Arith<T>::sub(F[k], v); });
-      __syncthreads();
-      const LevelGeo<T>& Lc = geo[l + 1];
-      T* Fc = sm + D->sm_f[l + 1];
-      const int tr = D->transfer[l];
-      for (int k = tid; k < Lc.rows * Lc.cols; k += kTailSmemThreads) {
-        if (!tail_node(Lc, k, i, j)) continue;
-        Fc[k] = restrict_any<T, EXACT>(L, tr, Dd, i, j, SmemIdx());
+      if (!res) {
+        flip ^= 1ull << l;
+      } else {  // z: the coarse level starts from 0
+        __syncthreads();
+        const LevelGeo<T>& Lc = geo[l + 1];
+        T* Fc = sm + D->sm_f[l + 1];
+        const int tr = D->transfer[l];
+        each(Lc, [&](int k, int i, int j) {
+          const T v = restrict_any<T, EXACT>(L, tr, sm + cb, i, j);
+          Fc[k] = v;
+          if (op.z) start_at(l + 1, k, i, j, v);
+        });
       }
     } else if (op.x == kOpCoarsest) {
       T* U = sm + cur(l);
-      if (D->dense.m > 0) {
-        T* fv = reinterpret_cast<T*>(tail_smem + TailSmem<T>::stage(D->sm_elems));
-        dense_coarse_vec<T, EXACT>(D->dense, L, F, fv, U, SmemIdx(), tid, kTailSmemThreads);
-      } else if (tid == 0) {
-        const int c = D->coarsest_zero ? smem_idx(L, 0, 0) : smem_idx(L, 1, 1);
-        U[c] = D->coarsest_zero ? T(0) : Arith<T>::div(F[c], D->coarsest_a);
-      }
+      if (D->dense.m > 0)
+        dense_coarse_vec<T, EXACT>(D->dense, L, F, reinterpret_cast<T*>(tail_smem + tail_scratch<T>(D->sm_elems, nst)), U,
+                                   GlobalIdx(), tid, kTailSmemThreads);
+      else if (tid == 0)
+        U[D->coarsest_idx] = D->coarsest_zero ? T(0) : Arith<T>::div(F[D->coarsest_idx], D->coarsest_a);
     } else {  // kOpProlong
       const LevelGeo<T>& Lc = geo[l + 1];
       const T* V = sm + cur(l + 1);
       T* U = sm + cur(l);
       const int tr = D->transfer[l];
-      for (int k = tid; k < total; k += kTailSmemThreads) {
-        if (!tail_node(L, k, i, j)) continue;
-        const T e = prolong_any<T, EXACT>(Lc, tr, V, i, j, SmemIdx());
-        U[k] = Arith<T>::add(U[k], e);
-      }
+      each(L, [&](int k, int i, int j) { U[k] = Arith<T>::add(U[k], prolong_any<T, EXACT>(Lc, tr, V, i, j)); });
     }
     __syncthreads();
   }
   {  // top level: u back to global memory (interior nodes)
-    const LevelGeo<T>& L = geo[top];
     const int c = cur(top);
-    for (int k = tid; k < L.rows * L.cols; k += kTailSmemThreads) {
-      int i, j;
-      if (!tail_node(L, k, i, j)) continue;
-      D->u[top][(int64_t)j * L.pitch + (k - j * L.cols)] = sm[c + k];
-    }
+    each(geo[top], [&](int k, int, int) { D->u[top][k] = sm[c + k]; });
   }
 }
 
@@ -1738,6 +1803,32 @@ int gen_block_rows(const LevelDev<T>& L, unsigned gx) {
   return by;
 }
 
+// Launch with programmatic dependent launch (device.cuh) if the grid has at most `limit`
+// threads per SM: the kernel's start and its reads of level tables then overlap the kernel
+// before it. Measured on GB300: 200 dependent empty kernels in a graph take 0.85 us each
+// without and 0.66 with; whole solves, limit 0 / 128 / 1024: FP64 128^2 2.18 / 1.75 / 1.89 ms,
+// FP64 periodic 512^2 3.98 / 3.46 / 4.35; limit 0 / 512 / 4096: mixed 256^2 1.30 / 1.06 /
+// 1.07, mixed 4096^2 10.37 / 9.65 / 9.54. FP64 stops at one warp to each FP64 unit (128
+// threads per SM): blocks that start early fill whatever SMs have room, and two warps on
+// one unit while others idle cost more than the start saves.
+template <typename T>
+constexpr int kPdlThreadsPerSm = sizeof(T) == 8 ? 128 : 4096;
+
+template <typename T, typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  const int64_t threads = (int64_t)grid.x * grid.y * block.x * block.y;
+  cfg.numAttrs = threads <= (int64_t)kPdlThreadsPerSm<T> * sm_count() ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Whether every node of a launch goes to the octets (rows.cuh), the fast ones too: small
 // levels, where their shorter chains beat one thread per node as long as the octets' warps
 // leave room on the FP64 units (kOctetWarpsPerUnit warps to each of an SM's four).
@@ -1751,19 +1842,17 @@ bool all_octets(const LevelGeo<T>& L, int colour) {
 // Launch arguments of a half-sweep (colour red or black) or residual (all nodes): `wx` fast
 // nodes' columns of blocks, `rows` storage rows per block of `by` warps.
 template <typename T>
-SweepArgs<T> sweep_args(const LevelPair<T>& L, int colour, int gx, int rows, int by, dim3& grid, size_t& smem) {
+SweepArgs<T> sweep_args(const LevelPair<T>& L, int colour, int gx, int rows, int by, dim3& grid) {
   SweepArgs<T> A;
   A.L = L.h;
   A.Lp = L.d;
   A.S = make_strips<T>(L.h, colour, all_octets<T>(L.h, colour));
   A.colour = colour;
-  A.K = oct_slots(L.h.maxcnt);
   A.gx = gx;
   A.sblocks = (A.S.total + 4 * by - 1) / (4 * by);
   const int gy = (L.h.rows + rows - 1) / rows;
   // a residual with no fast nodes needs no other blocks (a half-sweep's copy the other colour)
   grid = dim3(A.sblocks + (A.S.all && colour == kAllNodes ? 0 : gx * gy));
-  smem = A.sblocks > 0 ? 4 * by * oct_bytes<T>(A.K) : 0;
   return A;
 }
 
@@ -1773,15 +1862,14 @@ cudaError_t launch_half_sweep_nt(const LevelPair<T>& L, bool exact, const T* uin
   int gx = (L.h.cols + kBX - 1) / kBX;
   if (L.h.kind == kAxis) gx = ((L.h.n + 2) / 2 + kBX - 1) / kBX;  // pairs (2p, 2p+1), 2p <= n
   dim3 g;
-  size_t sm;
-  const SweepArgs<T> A = sweep_args(L, red, gx, kBY * RowsPer<T>::value, kBY, g, sm);
+  const SweepArgs<T> A = sweep_args(L, red, gx, kBY * RowsPer<T>::value, kBY, g);
   const dim3 b(kBX, kBY);
   if (L.h.per) {
-    if (exact) k_half_sweep_nt<T, true, NT, true><<<g, b, sm, s>>>(A, uin, f, uout);
-    else k_half_sweep_nt<T, false, NT, true><<<g, b, sm, s>>>(A, uin, f, uout);
+    if (exact) return launch_pdl<T>(k_half_sweep_nt<T, true, NT, true>, g, b, s, A, uin, f, uout);
+    else return launch_pdl<T>(k_half_sweep_nt<T, false, NT, true>, g, b, s, A, uin, f, uout);
   } else {
-    if (exact) k_half_sweep_nt<T, true, NT, false><<<g, b, sm, s>>>(A, uin, f, uout);
-    else k_half_sweep_nt<T, false, NT, false><<<g, b, sm, s>>>(A, uin, f, uout);
+    if (exact) return launch_pdl<T>(k_half_sweep_nt<T, true, NT, false>, g, b, s, A, uin, f, uout);
+    else return launch_pdl<T>(k_half_sweep_nt<T, false, NT, false>, g, b, s, A, uin, f, uout);
   }
   return cudaGetLastError();
 }
@@ -1796,16 +1884,15 @@ cudaError_t launch_half_sweep(const LevelPair<T>& L, bool exact, const T* uin, c
   if (L.h.kind == kAxis) gx = ((L.h.n + 2) / 2 + kBX - 1) / kBX;  // pairs (2p, 2p+1), 2p <= n
   const int by = gen_block_rows(L.h, gx);
   dim3 g;
-  size_t sm;
-  const SweepArgs<T> A = sweep_args(L, red, gx, by, by, g, sm);
+  const SweepArgs<T> A = sweep_args(L, red, gx, by, by, g);
   const dim3 b(kBX, by);
   const bool deep = sizeof(T) == 4 && L.h.rows < kGenDeepRows;
   if (deep) {
-    if (exact) k_half_sweep_gen<T, true, true><<<g, b, sm, s>>>(A, uin, f, uout);
-    else k_half_sweep_gen<T, false, true><<<g, b, sm, s>>>(A, uin, f, uout);
+    if (exact) return launch_pdl<T>(k_half_sweep_gen<T, true, true>, g, b, s, A, uin, f, uout);
+    else return launch_pdl<T>(k_half_sweep_gen<T, false, true>, g, b, s, A, uin, f, uout);
   } else {
-    if (exact) k_half_sweep_gen<T, true, false><<<g, b, sm, s>>>(A, uin, f, uout);
-    else k_half_sweep_gen<T, false, false><<<g, b, sm, s>>>(A, uin, f, uout);
+    if (exact) return launch_pdl<T>(k_half_sweep_gen<T, true, false>, g, b, s, A, uin, f, uout);
+    else return launch_pdl<T>(k_half_sweep_gen<T, false, false>, g, b, s, A, uin, f, uout);
   }
   return cudaGetLastError();
 }
@@ -1857,16 +1944,15 @@ cudaError_t launch_apply(const LevelPair<T>& L, bool exact, const T* u, T* out, 
 template <typename T, int NT>
 cudaError_t launch_residual_nt(const LevelPair<T>& L, bool exact, const T* u, const T* f, T* d, cudaStream_t s) {
   dim3 g;
-  size_t sm;
   const SweepArgs<T> A =
-      sweep_args(L, kAllNodes, (L.h.cols + kBX - 1) / kBX, kBY * RowsPer<T>::value, kBY, g, sm);
+      sweep_args(L, kAllNodes, (L.h.cols + kBX - 1) / kBX, kBY * RowsPer<T>::value, kBY, g);
   const dim3 b(kBX, kBY);
   if (L.h.per) {
-    if (exact) k_residual_nt<T, true, NT, true><<<g, b, sm, s>>>(A, u, f, d);
-    else k_residual_nt<T, false, NT, true><<<g, b, sm, s>>>(A, u, f, d);
+    if (exact) return launch_pdl<T>(k_residual_nt<T, true, NT, true>, g, b, s, A, u, f, d);
+    else return launch_pdl<T>(k_residual_nt<T, false, NT, true>, g, b, s, A, u, f, d);
   } else {
-    if (exact) k_residual_nt<T, true, NT, false><<<g, b, sm, s>>>(A, u, f, d);
-    else k_residual_nt<T, false, NT, false><<<g, b, sm, s>>>(A, u, f, d);
+    if (exact) return launch_pdl<T>(k_residual_nt<T, true, NT, false>, g, b, s, A, u, f, d);
+    else return launch_pdl<T>(k_residual_nt<T, false, NT, false>, g, b, s, A, u, f, d);
   }
   return cudaGetLastError();
 }
@@ -1880,16 +1966,15 @@ cudaError_t launch_residual(const LevelPair<T>& L, bool exact, const T* u, const
   const int gx = (L.h.cols + kBX - 1) / kBX;
   const int by = gen_block_rows(L.h, gx);
   dim3 g;
-  size_t sm;
-  const SweepArgs<T> A = sweep_args(L, kAllNodes, gx, by, by, g, sm);
+  const SweepArgs<T> A = sweep_args(L, kAllNodes, gx, by, by, g);
   const dim3 b(kBX, by);
   const bool deep = sizeof(T) == 4 && L.h.rows < kGenDeepRows;
   if (deep) {
-    if (exact) k_residual_gen<T, true, true><<<g, b, sm, s>>>(A, u, f, d);
-    else k_residual_gen<T, false, true><<<g, b, sm, s>>>(A, u, f, d);
+    if (exact) return launch_pdl<T>(k_residual_gen<T, true, true>, g, b, s, A, u, f, d);
+    else return launch_pdl<T>(k_residual_gen<T, false, true>, g, b, s, A, u, f, d);
   } else {
-    if (exact) k_residual_gen<T, true, false><<<g, b, sm, s>>>(A, u, f, d);
-    else k_residual_gen<T, false, false><<<g, b, sm, s>>>(A, u, f, d);
+    if (exact) return launch_pdl<T>(k_residual_gen<T, true, false>, g, b, s, A, u, f, d);
+    else return launch_pdl<T>(k_residual_gen<T, false, false>, g, b, s, A, u, f, d);
   }
   return cudaGetLastError();
 }
@@ -1901,7 +1986,7 @@ cudaError_t launch_restrict(const LevelPair<T>& Lf, const LevelPair<T>& Lc, int 
   const dim3 b(kBX, kBY);
   if (transfer != kStandardCubic && Lc.h.rows >= kTransferRowsMinLevelRows) {
     g.y = (Lc.h.rows + kBY * kTransferRows - 1) / (kBY * kTransferRows);
-#define NSMG_RESTRICT(E, P) k_restrict<T, E, P, kTransferRows><<<g, b, 0, s>>>(Lf.d, Lc.d, transfer, d, fc, tc)
+#define NSMG_RESTRICT(E, P) k_restrict<T, E, P, kTransferRows><<<g, b, 0, s>>>(Lf.h, Lc.h, transfer, d, fc, tc)
     if (Lf.h.per) {
       if (exact) NSMG_RESTRICT(true, true);
       else NSMG_RESTRICT(false, true);
@@ -1914,18 +1999,18 @@ cudaError_t launch_restrict(const LevelPair<T>& Lf, const LevelPair<T>& Lc, int 
   }
   if (transfer == kStandardCubic) {
     if (Lf.h.per) {
-      if (exact) k_restrict_cubic<T, true, true><<<g, b, 0, s>>>(Lf.d, Lc.d, d, fc, tc);
-      else k_restrict_cubic<T, false, true><<<g, b, 0, s>>>(Lf.d, Lc.d, d, fc, tc);
+      if (exact) return launch_pdl<T>(k_restrict_cubic<T, true, true>, g, b, s, Lf.h, Lc.h, d, fc, tc);
+      else return launch_pdl<T>(k_restrict_cubic<T, false, true>, g, b, s, Lf.h, Lc.h, d, fc, tc);
     } else {
-      if (exact) k_restrict_cubic<T, true, false><<<g, b, 0, s>>>(Lf.d, Lc.d, d, fc, tc);
-      else k_restrict_cubic<T, false, false><<<g, b, 0, s>>>(Lf.d, Lc.d, d, fc, tc);
+      if (exact) return launch_pdl<T>(k_restrict_cubic<T, true, false>, g, b, s, Lf.h, Lc.h, d, fc, tc);
+      else return launch_pdl<T>(k_restrict_cubic<T, false, false>, g, b, s, Lf.h, Lc.h, d, fc, tc);
     }
   } else if (Lf.h.per) {
-    if (exact) k_restrict<T, true, true, 1><<<g, b, 0, s>>>(Lf.d, Lc.d, transfer, d, fc, tc);
-    else k_restrict<T, false, true, 1><<<g, b, 0, s>>>(Lf.d, Lc.d, transfer, d, fc, tc);
+    if (exact) return launch_pdl<T>(k_restrict<T, true, true, 1>, g, b, s, Lf.h, Lc.h, transfer, d, fc, tc);
+    else return launch_pdl<T>(k_restrict<T, false, true, 1>, g, b, s, Lf.h, Lc.h, transfer, d, fc, tc);
   } else {
-    if (exact) k_restrict<T, true, false, 1><<<g, b, 0, s>>>(Lf.d, Lc.d, transfer, d, fc, tc);
-    else k_restrict<T, false, false, 1><<<g, b, 0, s>>>(Lf.d, Lc.d, transfer, d, fc, tc);
+    if (exact) return launch_pdl<T>(k_restrict<T, true, false, 1>, g, b, s, Lf.h, Lc.h, transfer, d, fc, tc);
+    else return launch_pdl<T>(k_restrict<T, false, false, 1>, g, b, s, Lf.h, Lc.h, transfer, d, fc, tc);
   }
   return cudaGetLastError();
 }
@@ -1937,7 +2022,7 @@ cudaError_t launch_prolong_add(const LevelPair<T>& Lf, const LevelPair<T>& Lc, i
   const T* ui = uin ? uin : uf;
   if (transfer != kStandardCubic && Lf.h.kind == kAxis && Lf.h.rows >= kTransferRowsMinLevelRows) {
     const dim3 g((Lf.h.n / 2 + 1 + kBX - 1) / kBX, (Lf.h.rows + kBY * kTransferRows - 1) / (kBY * kTransferRows));
-#define NSMG_PROLONG(E, P) k_prolong_add<T, E, P, kTransferRows, true><<<g, b, 0, s>>>(Lf.d, Lc.d, transfer, ui, uf, vc)
+#define NSMG_PROLONG(E, P) k_prolong_add<T, E, P, kTransferRows, true><<<g, b, 0, s>>>(Lf.h, Lc.h, transfer, ui, uf, vc)
     if (Lc.h.per) {
       if (exact) NSMG_PROLONG(true, true);
       else NSMG_PROLONG(false, true);
@@ -1951,18 +2036,18 @@ cudaError_t launch_prolong_add(const LevelPair<T>& Lf, const LevelPair<T>& Lc, i
   const dim3 g = grid_of(Lf.h);
   if (transfer == kStandardCubic) {
     if (Lc.h.per) {
-      if (exact) k_prolong_cubic<T, true, true><<<g, b, 0, s>>>(Lf.d, Lc.d, ui, uf, vc);
-      else k_prolong_cubic<T, false, true><<<g, b, 0, s>>>(Lf.d, Lc.d, ui, uf, vc);
+      if (exact) return launch_pdl<T>(k_prolong_cubic<T, true, true>, g, b, s, Lf.h, Lc.h, ui, uf, vc);
+      else return launch_pdl<T>(k_prolong_cubic<T, false, true>, g, b, s, Lf.h, Lc.h, ui, uf, vc);
     } else {
-      if (exact) k_prolong_cubic<T, true, false><<<g, b, 0, s>>>(Lf.d, Lc.d, ui, uf, vc);
-      else k_prolong_cubic<T, false, false><<<g, b, 0, s>>>(Lf.d, Lc.d, ui, uf, vc);
+      if (exact) return launch_pdl<T>(k_prolong_cubic<T, true, false>, g, b, s, Lf.h, Lc.h, ui, uf, vc);
+      else return launch_pdl<T>(k_prolong_cubic<T, false, false>, g, b, s, Lf.h, Lc.h, ui, uf, vc);
     }
   } else if (Lc.h.per) {
-    if (exact) k_prolong_add<T, true, true, 1, false><<<g, b, 0, s>>>(Lf.d, Lc.d, transfer, ui, uf, vc);
-    else k_prolong_add<T, false, true, 1, false><<<g, b, 0, s>>>(Lf.d, Lc.d, transfer, ui, uf, vc);
+    if (exact) return launch_pdl<T>(k_prolong_add<T, true, true, 1, false>, g, b, s, Lf.h, Lc.h, transfer, ui, uf, vc);
+    else return launch_pdl<T>(k_prolong_add<T, false, true, 1, false>, g, b, s, Lf.h, Lc.h, transfer, ui, uf, vc);
   } else {
-    if (exact) k_prolong_add<T, true, false, 1, false><<<g, b, 0, s>>>(Lf.d, Lc.d, transfer, ui, uf, vc);
-    else k_prolong_add<T, false, false, 1, false><<<g, b, 0, s>>>(Lf.d, Lc.d, transfer, ui, uf, vc);
+    if (exact) return launch_pdl<T>(k_prolong_add<T, true, false, 1, false>, g, b, s, Lf.h, Lc.h, transfer, ui, uf, vc);
+    else return launch_pdl<T>(k_prolong_add<T, false, false, 1, false>, g, b, s, Lf.h, Lc.h, transfer, ui, uf, vc);
   }
   return cudaGetLastError();
 }
@@ -1971,15 +2056,14 @@ template <typename T>
 cudaError_t launch_coarsest_dense(const DenseCoarse<T>& C, const LevelPair<T>& L, bool exact, const T* f, T* u,
                                   cudaStream_t s) {
   const int threads = std::min(1024, (C.m + 31) / 32 * 32);
-  if (exact) k_coarsest_dense<T, true><<<1, threads, 0, s>>>(C, L.h, f, u);
-  else k_coarsest_dense<T, false><<<1, threads, 0, s>>>(C, L.h, f, u);
+  if (exact) return launch_pdl<T>(k_coarsest_dense<T, true>, 1, threads, s, C, L.h, f, u);
+  else return launch_pdl<T>(k_coarsest_dense<T, false>, 1, threads, s, C, L.h, f, u);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_coarsest(int64_t idx, T a, int zero_mean, const T* f, T* u, cudaStream_t s) {
-  k_coarsest<T><<<1, 32, 0, s>>>(idx, a, zero_mean, f, u);
-  return cudaGetLastError();
+  return launch_pdl<T>(k_coarsest<T>, 1, 32, s, idx, a, zero_mean, f, u);
 }
 
 // Blocks of a kernel resident on the whole GPU at once (256-thread blocks), looked up
@@ -2017,8 +2101,7 @@ cudaError_t launch_resnorm(const LevelPair<T>& L, bool exact, const T* u, const 
 
 template <typename T>
 cudaError_t launch_first_half_zero(const LevelPair<T>& L, const T* f, T* t, int red, cudaStream_t s) {
-  k_first_half_zero<T><<<grid_of(L.h), dim3(kBX, kBY), 0, s>>>(L.d, f, t, red);
-  return cudaGetLastError();
+  return launch_pdl<T>(k_first_half_zero<T>, grid_of(L.h), dim3(kBX, kBY), s, L.h, f, t, red);
 }
 
 template <typename T, bool EXACT, int NT>
@@ -2200,25 +2283,16 @@ cudaError_t launch_batch_ir_update(const BatchLevel<double>* entries, const int*
 }
 
 template <typename T>
-TailSmemPlan tail_smem_plan(int sm_elems, int maxcnt, int dense_m) {
-  TailSmemPlan P;
-  P.K = oct_slots(maxcnt);
-  const size_t base = TailSmem<T>::stage(sm_elems), per_warp = 4 * oct_bytes<T>(P.K);
-  const size_t room = base < kTailSmemMaxBytes ? kTailSmemMaxBytes - base : 0;
-  const size_t warps = std::min<size_t>(kTailSmemThreads / 32, room / per_warp);
-  P.octs = 4 * (int)warps;
-  P.bytes = base + std::max(warps * per_warp, 2 * (size_t)dense_m * sizeof(T));
-  if (warps == 0 || P.bytes > kTailSmemMaxBytes) P.octs = 0;
-  return P;
+size_t tail_smem_bytes(int sm_elems, int nst, int dense_m) {
+  return tail_scratch<T>(sm_elems, nst) + 2 * (size_t)dense_m * sizeof(T);
 }
 
 template <typename T>
-cudaError_t launch_tail_smem(const TailDesc<T>* desc, size_t bytes, const int4* prog, int nops, bool exact,
+cudaError_t launch_tail_smem(const TailDesc<T>* desc, size_t bytes, const int4* prog, int nops, int zero, bool exact,
                              cudaStream_t s) {
-  const void* fn = exact ? (const void*)k_tail_smem<T, true> : (const void*)k_tail_smem<T, false>;
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (exact) k_tail_smem<T, true><<<1, kTailSmemThreads, bytes, s>>>(desc, prog, nops);
-  else k_tail_smem<T, false><<<1, kTailSmemThreads, bytes, s>>>(desc, prog, nops);
+  const auto fn = exact ? k_tail_smem<T, true> : k_tail_smem<T, false>;
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmemMaxBytes);
+  fn<<<1, kTailSmemThreads, bytes, s>>>(desc, prog, nops, zero);
   return cudaGetLastError();
 }
 
@@ -2249,9 +2323,9 @@ cudaError_t launch_tail_smem(const TailDesc<T>* desc, size_t bytes, const int4* 
   template cudaError_t launch_copy_boundary<T>(const LevelPair<T>&, const T*, T*, cudaStream_t);      \
   template cudaError_t launch_batch_step<T>(int, const BatchLevel<T>*, const int*, int, int, int, const int*, bool, \
                                             cudaStream_t);                                             \
+  template cudaError_t launch_tail_smem<T>(const TailDesc<T>*, size_t, const int4*, int, int, bool, cudaStream_t); \
+  template size_t tail_smem_bytes<T>(int, int, int);                                                  \
   template int tail_ctas<T>(bool);                                                                    \
-  template cudaError_t launch_tail_smem<T>(const TailDesc<T>*, size_t, const int4*, int, bool, cudaStream_t); \
-  template TailSmemPlan tail_smem_plan<T>(int, int, int);                                             \
   template cudaError_t launch_tail<T>(int, const TailDesc<T>*, const int4*, int, bool, cudaStream_t);
 
 NSMG_INSTANTIATE(double)

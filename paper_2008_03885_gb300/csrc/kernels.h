@@ -94,7 +94,7 @@ cudaError_t launch_ir_residual(const LevelPair<double>& L, bool exact, const dou
 cudaError_t launch_ir_update(const LevelPair<double>& L, const LevelPair<float>& L32, double* u, const float* e,
                              double inv_scale, cudaStream_t s);
 
-// ---- small-level tail: one thread block runs a whole sub-cycle ---------------
+// ---- small-level tail: one thread block or cluster runs a whole sub-cycle ------
 constexpr int kTailMaxLevels = 40;
 // kOpSmooth with z = 1: the first red-black sweep from u = 0 (the level's u is not zeroed
 // first; its red half-sweep needs no stencil).
@@ -114,30 +114,28 @@ struct TailDesc {
   T coarsest_a;
   int32_t coarsest_zero;  // periodic single node: the zero-mean solution 0
   DenseCoarse<T> dense;   // m > 0: the coarsest level's dense solve
-  // shared-memory-resident variant: per level, element offsets of u, t, f, d in the
-  // block's shared memory (compact rows x cols layout) and the number of levels held
-  int32_t sm_u[kTailMaxLevels], sm_t[kTailMaxLevels], sm_f[kTailMaxLevels], sm_d[kTailMaxLevels];
+  // shared-memory-resident variant: per level, element offsets of u, t, f in the
+  // block's shared memory (storage layout; the residual goes to the one of u and t that
+  // is not current)
+  int32_t sm_u[kTailMaxLevels], sm_t[kTailMaxLevels], sm_f[kTailMaxLevels];
   int32_t sm_top;     // first level held (the sub-cycle's top level)
   int32_t sm_elems;   // shared-memory elements of the level arrays
-  int32_t sm_octs, sm_K;  // octets at work and values staged by each (TailSmemPlan)
   int32_t nlev;       // levels of the hierarchy (those from sm_top on are held)
 };
 
-// The same op list, with every level from sm_top down held in one block's shared
-// memory (u and f of the top level are loaded at start, u written back at the end).
+// The same steps with every level from sm_top down held in one block's shared memory (f
+// and, unless `zero`, u of the top level are loaded at start, u written back at the end).
+// The op list differs from launch_tail's: kOpZero with z = 1 also does the first
+// half-sweep from u = 0 (zero = 1: the list starts with kOpZero), kOpResRestrict with
+// z = 1 does it for the coarse level, and kOpSmooth with z = 1 follows one of them.
 template <typename T>
-cudaError_t launch_tail_smem(const TailDesc<T>* desc, size_t bytes, const int4* prog, int nops, bool exact,
+cudaError_t launch_tail_smem(const TailDesc<T>* desc, size_t bytes, const int4* prog, int nops, int zero, bool exact,
                              cudaStream_t s);
-// Shared memory of the shared-memory tail: the level arrays (sm_elems values), then the
-// staging of as many octets as fit (rows of up to maxcnt terms), which the dense coarsest
-// solve (dense_m unknowns) reuses. octs = 0: does not fit kTailSmemMaxBytes.
-struct TailSmemPlan {
-  int octs = 0, K = 0;
-  size_t bytes = 0;
-};
+// Shared memory of that kernel: the level arrays (sm_elems values), the interior stencils
+// of its nst levels, and the vectors of the dense coarsest solve (dense_m unknowns).
 template <typename T>
-TailSmemPlan tail_smem_plan(int sm_elems, int maxcnt, int dense_m);
-constexpr size_t kTailSmemMaxBytes = 220 * 1024;  // leaves room for the kernel's static arrays
+size_t tail_smem_bytes(int sm_elems, int nst, int dense_m);
+constexpr size_t kTailSmemMaxBytes = 208 * 1024;  // leaves room for the kernel's static arrays (16 KB)
 
 // Run `nops` ops (x = TailOp, y = level) in order inside one thread-block cluster of
 // `ctas` CTAs, with a cluster barrier after each phase. Op semantics match the

@@ -29,6 +29,23 @@ struct __align__(16) ClassTerm {
   int32_t dx, dy;
 };
 
+// One group of equal coefficient of a class row: the coefficient and its cnt (0: no group)
+// terms in evaluation order, as three 16-byte loads. A class's records are `maxg`
+// (LevelGeo) consecutive ones, in group order. A term (dx, dy) is stored as
+//   4 (dy pitch + dx) + other   on axis levels,
+//   4 dy pitch + 2 dx + other   on rotated levels (column (i + dx) >> 1),
+// so that its storage offset from node (i, j) is (d + 2 (i & 1)) >> 2 on rotated levels
+// and d >> 2 on axis ones; other = 1 if the term has the other colour than the node.
+constexpr int kGroupMax = 8;
+template <typename T>
+struct __align__(16) GroupRec {
+  T c;
+  int32_t cnt;
+  int32_t pad[sizeof(T) == 8 ? 1 : 2];
+  int32_t d[kGroupMax];
+};
+static_assert(sizeof(GroupRec<double>) == 48 && sizeof(GroupRec<float>) == 48, "three 16-byte loads");
+
 // Device-resident description of one level in precision T.
 //
 // Points live on an integer lattice (i, j), 0 <= i, j <= n. Axis levels hold every
@@ -54,11 +71,13 @@ struct LevelGeo {
   int32_t kind, n, rows, cols, pitch;
   int32_t nt, rx, ry;
   int32_t small, clsw;
-  int32_t maxcnt;             // terms of the longest class row
+  int32_t maxg;               // groups of the class row with most (0: no group records, as
+                              // some group has more than kGroupMax terms)
   T wd;                       // omega / a_pp at fast nodes
   const int2* cls;            // per class: (first term, term count)
   const T* cls_wd;            // per class: omega / a_pp
   const ClassTerm<T>* terms;  // merged terms of every class
+  const GroupRec<T>* groups;  // the same rows as group records, maxg to a class
   int32_t bf16;  // FP32 inner levels: round every stored value to bfloat16 (storage trial)
   int32_t per;   // 1: periodic level (see above)
   int32_t lo;    // first unknown index: 1 - per

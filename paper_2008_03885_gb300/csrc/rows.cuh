@@ -1,23 +1,22 @@
 // Rows of boundary-class nodes by octets of lanes.
 //
-// A class row is a list of up to maxcnt (coefficient, offset) records, different for
-// neighbouring nodes. One thread per node walks it as a serial chain: record, value,
-// record, value, each waiting out an L2 latency, and in FP64 every divergent branch of a
-// warp pays the FP64 unit again (one warp instruction occupies it for 64 clocks on GB300,
-// however few lanes are active: measured 64.0 clocks with 1 as with 32 active lanes). Small
-// levels consist of such nodes alone, and the strips along the boundary of a large level
-// end up as the last warps of its grid.
+// A class row is a list of up to 45 (121 with cubic transfers) coefficients and offsets,
+// different for neighbouring nodes. One thread per node walks it as a serial chain:
+// record, value, record, value, each waiting out an L2 latency, and in FP64 every divergent
+// branch of a warp pays the FP64 unit again (one warp instruction occupies it for 64 clocks
+// on GB300, however few lanes are active: measured 64.0 clocks with 1 as with 32 active
+// lanes). Small levels consist of such nodes alone, and the strips along the boundary of a
+// large level end up as the last warps of its grid.
 //
-// Here eight lanes share a node: the row's records are fetched in one batch (six a lane
-// at 45 terms), then its values in a second, and staged in shared memory. In the exact
-// order each lane then sums whole groups of equal coefficient (groups g, g + 8, ... in
-// lane g: their sums are independent), and the group products are added in group order;
-// with FMA the terms are one ordered chain from shared memory. The operations and their
-// order are those of RowSum, so the results are the same bits; a 45-point FP64 row takes
-// about 20 warp instructions of FP64 instead of 60.
-//
-// Measured on GB300 (ncu, warm caches), FP64 half-sweeps of 45-point levels: 33^2 rotated
-// 18.7 us before; see kernels.cu for the figures after.
+// Here eight lanes share a node and each takes whole groups of equal coefficient (GroupRec:
+// coefficient and up to eight offsets in 48 bytes; groups g and g + 8 of the row in lane
+// g): one batch of record loads, one batch of value loads, then the group sums of all
+// lanes at once, and the group products added in group order by shuffles. With FMA the
+// row is one ordered chain, handed from lane to lane. The operations and their order are
+// those of RowSum, so the results are the same bits; a 45-point FP64 row takes about 20
+// warp instructions of FP64 instead of 60, and about 250 instructions in all (a lone warp
+// spends 8-16 clocks on each). A first form that staged records and values in shared
+// memory and summed from there took 600 instructions; see kernels.cu for both timings.
 #pragma once
 
 #include "device.cuh"
@@ -26,13 +25,6 @@ namespace nsmg {
 namespace {
 
 constexpr int kOct = 8;  // lanes per node
-
-// Staging of one octet's row in shared memory: K values, K coefficients, K group starts.
-template <typename T>
-__host__ __device__ constexpr size_t oct_bytes(int K) {
-  return (size_t)K * (2 * sizeof(T) + 1);
-}
-__host__ __device__ constexpr int oct_slots(int maxcnt) { return (maxcnt + kOct - 1) / kOct * kOct; }
 
 // The nodes of one colour (or of all colours) that the octets of a launch take: rows of
 // the lattice in three runs (below, above and beside the fast rectangle), each row cut
@@ -44,12 +36,14 @@ struct StripGeo {
   int32_t fB, cB;               // rows beside the fast rectangle
   int32_t wA, wL, wR;           // slots of a full row, left and right of the rectangle
   int32_t total;                // slots
+  uint32_t mA, mB;              // ceil(2^32 / wA), ceil(2^32 / (wL + wR)): slot / w = slot m >> 32
+                                // (exact for slot w < 2^32; w = 1 is handled apart)
 };
 
 enum RowColour : int { kBlackNodes = 0, kRedNodes = 1, kAllNodes = 2 };
 
 template <typename T>
-inline StripGeo make_strips(const LevelGeo<T>& L, int colour, bool all) {
+__host__ __device__ inline StripGeo make_strips(const LevelGeo<T>& L, int colour, bool all) {
   StripGeo S;
   const int lo = L.lo, hi = L.n - 1;
   const bool none = (all && !L.bdata) || L.fxe < L.rx || L.fye < L.ry;
@@ -68,6 +62,9 @@ inline StripGeo make_strips(const LevelGeo<T>& L, int colour, bool all) {
   S.wL = slots(lo, L.rx - 1);
   S.wR = slots(L.fxe + 1, hi);
   S.total = (S.cA0 + S.cA1) * S.wA + S.cB * (S.wL + S.wR);
+  auto magic = [](uint32_t w) { return w > 1 ? 0xffffffffu / w + 1 : 0u; };
+  S.mA = magic(S.wA);
+  S.mB = magic(S.wL + S.wR);
   return S;
 }
 
@@ -79,7 +76,7 @@ __device__ __forceinline__ bool strip_node(const LevelGeo<T>& L, const StripGeo&
   const int nA = (S.cA0 + S.cA1) * S.wA;
   int a, b, s;
   if (slot < nA) {
-    const int r = slot / S.wA;
+    const int r = S.mA ? (int)__umulhi((uint32_t)slot, S.mA) : slot;
     s = slot - r * S.wA;
     j = r < S.cA0 ? S.fA0 + r * S.rstep : S.fA1 + (r - S.cA0) * S.rstep;
     a = L.lo;
@@ -87,7 +84,7 @@ __device__ __forceinline__ bool strip_node(const LevelGeo<T>& L, const StripGeo&
   } else {
     const int w = S.wL + S.wR;
     slot -= nA;
-    const int r = slot / w;
+    const int r = S.mB ? (int)__umulhi((uint32_t)slot, S.mB) : slot;
     s = slot - r * w;
     j = S.fB + r * S.rstep;
     if (s < S.wL) {
@@ -108,105 +105,129 @@ __device__ __forceinline__ bool strip_node(const LevelGeo<T>& L, const StripGeo&
   return i <= b;
 }
 
-// (L u)(i, j) by the octet this lane belongs to, in every lane of it. All 32 lanes of the
-// warp call it together; `on` is uniform over an octet (off: cnt = 0, result 0). `at(i, j)`
-// gives the position of a node in u; `stage` is the octet's shared memory (oct_bytes(K),
-// K >= the row's term count). PB: records a lane fetches per batch.
-template <typename T, bool EXACT, int PB, class At>
-__device__ __forceinline__ T octet_row(const LevelGeo<T>& L, const T* __restrict__ u, bool on, int i, int j, int cl,
-                                       unsigned char* stage, int K, At at) {
-  const int lane = threadIdx.x & 31, l8 = lane & 7, sh = lane & 24;
-  T* xs = reinterpret_cast<T*>(stage);
-  T* cs = xs + K;
-  uint8_t* gs = reinterpret_cast<uint8_t*>(cs + K);
-  int2 e = make_int2(0, 0);
-  if (on) e = __ldg(&L.cls[cl]);
+// Row of class cl at (i, j), term by term in one thread: rows without group records, and
+// FP32 levels in shared memory.
+template <typename T, bool EXACT>
+__device__ __forceinline__ T serial_row(const LevelGeo<T>& L, const T* own, const T* opp, int i, int j, int cl) {
+  RowSum<T, EXACT> acc;
+  const int2 e = __ldg(&L.cls[cl]);
   const ClassTerm<T>* tt = L.terms + e.x;
-  const int cnt = e.y;
-  const int wmax = __reduce_max_sync(0xffffffffu, cnt);
-  int ng = 0;
-  for (int k0 = 0; k0 < wmax; k0 += kOct * PB) {
-    Term<T> t[PB];
-    T x[PB];
-#pragma unroll
-    for (int p = 0; p < PB; ++p) {
-      const int k = k0 + kOct * p + l8;
-      t[p].start = false;
-      if (k < cnt) t[p] = load_term(tt + k);
-    }
-#pragma unroll
-    for (int p = 0; p < PB; ++p) {
-      const int k = k0 + kOct * p + l8;
-      if (k < cnt) x[p] = u[at(i + t[p].dx, j + t[p].dy)];
-    }
-#pragma unroll
-    for (int p = 0; p < PB; ++p) {
-      const int k = k0 + kOct * p + l8;
-      if (k < cnt) {
-        xs[k] = x[p];
-        cs[k] = t[p].c;
-      }
-      if (EXACT) {
-        const unsigned m = (__ballot_sync(0xffffffffu, t[p].start) >> sh) & 0xffu;
-        if (t[p].start) gs[ng + __popc(m & ((1u << l8) - 1u))] = (uint8_t)k;
-        ng += __popc(m);
-      }
-    }
-  }
-  __syncwarp();
-  T s = T(0);
-  if (EXACT) {
-    for (int g = l8; g < ng; g += kOct) {
-      const int k0 = gs[g], k1 = g + 1 < ng ? gs[g + 1] : cnt;
-      T v = xs[k0];
+  const int at = (int)sidx(L, i, j);
+  const int other_at = (int)(opp - own), rot = L.kind == kRot;
 #pragma unroll 4
-      for (int k = k0 + 1; k < k1; ++k) v = Arith<T>::add(v, xs[k]);
-      xs[k0] = Arith<T>::mul(cs[k0], v);
-    }
-    __syncwarp();
-    if (ng > 0) s = xs[0];
-#pragma unroll 4
-    for (int g = 1; g < ng; ++g) s = Arith<T>::add(s, xs[gs[g]]);
-  } else {
-    if (cnt > 0) s = Arith<T>::mul(cs[0], xs[0]);
-#pragma unroll 8
-    for (int k = 1; k < cnt; ++k) s = Arith<T>::fma(cs[k], xs[k], s);
+  for (int k = 0; k < e.y; ++k) {
+    const Term<T> t = load_term(tt + k);
+    const int other = (rot ? t.dy : t.dx + t.dy) & 1;
+    acc.add(t.c, own[(int)sidx(L, i + t.dx, j + t.dy) - at + (other ? other_at : 0)], t.start);
   }
-  __syncwarp();  // the stage may be reused
-  return s;
+  return acc.value();
 }
 
-struct LevelAt {  // positions in a level's global storage
-  int kind, pitch;
-  __device__ __forceinline__ int64_t operator()(int i, int j) const {
-    return (int64_t)j * pitch + (kind == kRot ? (i >> 1) : i);
+template <typename T>
+__device__ __forceinline__ GroupRec<T> load_group(const GroupRec<T>* p) {
+  union {
+    int4 w[3];
+    GroupRec<T> r;
+  } v;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) v.w[k] = __ldg(reinterpret_cast<const int4*>(p) + k);
+  return v.r;
+}
+
+// (L u)(i, j) by the octet this lane belongs to, in every lane of it. All 32 lanes of the
+// warp call it together; `on` is uniform over an octet (off: some value). `own` and `opp`
+// point at the node's position in the arrays that hold the values of its own and of the
+// other colour (usually the same array). NREC: records a lane fetches at once. pre() runs
+// after the first records' loads and before any value is read.
+template <typename T, bool EXACT, int NREC, class Pre>
+__device__ __forceinline__ T octet_row(const LevelGeo<T>& L, const T* own, const T* opp, bool on, int i, int j, int cl,
+                                       Pre pre) {
+  if (L.maxg == 0) {
+    pre();
+    return on ? serial_row<T, EXACT>(L, own, opp, i, j, cl) : T(0);
   }
-};
+  const int l8 = threadIdx.x & 7, par2 = L.kind == kRot ? 2 * (i & 1) : 0;
+  const GroupRec<T>* R = L.groups + (int64_t)cl * L.maxg;
+  const bool split = own != opp;
+  T s = T(-0.0);  // the identity of both sums: x + (-0) = x, fma(c, x, -0) = fl(c x)
+  for (int g0 = 0; g0 < L.maxg; g0 += kOct * NREC) {
+    GroupRec<T> r[NREC];
+    T x[NREC][kGroupMax];
+#pragma unroll
+    for (int k = 0; k < NREC; ++k) {
+      const int g = g0 + kOct * k + l8;
+      r[k].cnt = 0;
+      r[k].c = T(1);
+      if (on && g < L.maxg) r[k] = load_group(R + g);
+    }
+    if (g0 == 0) pre();
+#pragma unroll
+    for (int k = 0; k < NREC; ++k) {
+      // a missing term adds -0 to either sum
+      const T pad = EXACT || r[k].c > T(0) ? T(-0.0) : T(0);
+#pragma unroll
+      for (int m = 0; m < kGroupMax; ++m) {
+        x[k][m] = pad;
+        if (m < r[k].cnt) x[k][m] = (split && (r[k].d[m] & 1) ? opp : own)[(r[k].d[m] + par2) >> 2];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < NREC; ++k) {
+      // most terms of a group and most groups of a row among the warp's octets
+      const int mx = __reduce_max_sync(0xffffffffu, r[k].cnt);
+      if (mx == 0) break;
+      const unsigned have = __ballot_sync(0xffffffffu, r[k].cnt > 0);
+      const int ng = 32 - __clz((have | have >> 8 | have >> 16 | have >> 24) & 0xffu);
+      if (EXACT) {
+        T p = x[k][0];
+#pragma unroll
+        for (int m = 1; m < kGroupMax; ++m)
+          if (m < mx) p = Arith<T>::add(p, x[k][m]);
+        p = r[k].cnt > 0 ? Arith<T>::mul(r[k].c, p) : T(-0.0);
+#pragma unroll
+        for (int t = 0; t < kOct; ++t)
+          if (t < ng) s = Arith<T>::add(s, __shfl_sync(0xffffffffu, p, t, kOct));
+      } else {
+#pragma unroll
+        for (int t = 0; t < kOct; ++t) {
+          if (t >= ng) break;
+          T v = s;
+#pragma unroll
+          for (int m = 0; m < 4; ++m) v = Arith<T>::fma(r[k].c, x[k][m], v);
+          if (mx > 4) {
+#pragma unroll
+            for (int m = 4; m < kGroupMax; ++m) v = Arith<T>::fma(r[k].c, x[k][m], v);
+          }
+          s = __shfl_sync(0xffffffffu, v, t, kOct);
+        }
+      }
+    }
+  }
+  return s;
+}
 
 enum RowMode : int { kRowRelax = 0, kRowResidual = 1 };
 
 // One slot per octet of block `bid`: half-sweep (out = relaxed value) or residual
 // (out = f - L u) of the strip nodes. blockDim = (32, warps).
-template <typename T, bool EXACT, int PB, int MODE>
+template <typename T, bool EXACT, int NREC, int MODE>
 __device__ __forceinline__ void strip_rows(const LevelGeo<T>& L, const StripGeo& S, int colour, int bid,
-                                           const T* __restrict__ u, const T* __restrict__ f, T* __restrict__ out,
-                                           unsigned char* smem, int K) {
+                                           const T* u, const T* f, T* out) {
   const int lane = threadIdx.x & 31, oct = threadIdx.y * 4 + (lane >> 3);
   const int slot = bid * (blockDim.y * 4) + oct;
   int i = 0, j = 0;
   const bool on = strip_node(L, S, colour, slot, i, j);
-  const LevelAt pos{L.kind, L.pitch};
-  const int64_t at = pos(i, j);
+  const int64_t at = sidx(L, i, j);
   const int cl = on ? class_of(L, i, j) : 0;
-  T fv = T(0), uv = T(0), wd = T(0);
-  if (on) {
-    fv = f[at];
-    if (MODE == kRowRelax) {
-      uv = u[at];
-      wd = L.cls_wd[cl];
+  T fv = T(0), uv = T(0);
+  const T wd = MODE == kRowRelax && on ? L.cls_wd[cl] : T(0);
+  const T s = octet_row<T, EXACT, NREC>(L, u + at, u + at, on, i, j, cl, [&]() {
+    pdl_wait();
+    if (on) {
+      fv = f[at];
+      if (MODE == kRowRelax) uv = u[at];
     }
-  }
-  const T s = octet_row<T, EXACT, PB>(L, u, on, i, j, cl, smem + oct * oct_bytes<T>(K), K, pos);
+  });
   if (!on || (lane & 7) != 0) return;
   const T r = Arith<T>::sub(fv, s);
   if (MODE == kRowRelax) out[at] = rnd(L, EXACT ? Arith<T>::add(uv, Arith<T>::mul(r, wd)) : Arith<T>::fma(r, wd, uv));

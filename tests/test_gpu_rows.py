@@ -83,3 +83,40 @@ def test_fma_order_stays_within_its_rounding_bound(n, order, co):
             assert np.all(np.abs(from_dev(h, l, out) - o.residual(l, u, f)) <= bound), l
     finally:
         h.close()
+
+
+def test_steps_in_a_caller_captured_graph_with_a_joined_stream():
+    """Small-level kernels start early (programmatic dependent launch): in a caller's graph
+    whose first step joins a second stream, and replayed on new data, they still see the
+    other stream's writes and give the bits of eager calls."""
+    n = 64
+    h = mg.mg_setup(n, 4, REDBLACK, GALERKIN)
+    try:
+        f = torch.tensor(synth.rhs_normal(n, 3), device="cuda")
+        src = torch.zeros_like(f)
+        u, d, u2, d2 = (torch.zeros_like(f) for _ in range(4))
+        fc, fc2 = mg.level_array(h, 1), mg.level_array(h, 1)
+        side, main = torch.cuda.Stream(), torch.cuda.Stream()
+        g = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g, stream=main):
+            side.wait_stream(main)
+            with torch.cuda.stream(side):
+                u.copy_(src)
+            main.wait_stream(side)
+            mg.mg_level_smooth(h, 0, u, f, 2, stream=main)
+            mg.mg_level_residual(h, 0, u, f, d, stream=main)
+            mg.mg_level_restrict(h, 0, d, fc, stream=main)
+            mg.mg_level_prolong_add(h, 0, u, fc, stream=main)
+        for seed in range(3):
+            src.copy_(torch.tensor(synth.rhs_normal(n, 7 + seed), device="cuda"))
+            g.replay()
+            u2.copy_(src)
+            mg.mg_level_smooth(h, 0, u2, f, 2)
+            mg.mg_level_residual(h, 0, u2, f, d2)
+            mg.mg_level_restrict(h, 0, d2, fc2)
+            mg.mg_level_prolong_add(h, 0, u2, fc2)
+            torch.cuda.synchronize()
+            assert torch.equal(u, u2) and torch.equal(d, d2) and torch.equal(fc, fc2), seed
+    finally:
+        h.close()
