@@ -1,0 +1,183 @@
+// The FP64 refinement residual r = f - L u of second-order levels in fixed point.
+//
+// GB300 has one FP64 unit of half a lane per clock to each SM quarter, so the residual of a
+// 5-point level (about ten FP64 operations a node) is bound by it, where its 20 bytes a node
+// need 200 us of HBM at 8193^2. Its 64-bit integer adds run 30 times as fast. The 5-point
+// operator is s = 1 / h^2 times the integers (-1; 4), so a tile's u values are written as
+// integers in units of 2^(E - 1081) (E: the largest biased exponent in the tile and its halo:
+// six bits below the last bit of the largest value), the stencil sum T is formed exactly,
+// and r = f - s T is one fused multiply-add; FP64 keeps two operations a node (that one and
+// the square for the norm).
+//
+// Precision. A value of exponent E or up to 6 below is exact; smaller ones are rounded to
+// half a unit, 2^-7 of the largest value's last bit, where FP64 rounds every partial sum (up
+// to 8 times the value) to half its own last bit. Mixed solves run to their floor keep a
+// relative residual of 0.45-0.5 of the FP64 sum's (8193^2: 9.3e-14 for 2.0e-13), and their
+// error against the exact discrete solution falls from 1e-14-3e-13 to 5e-16-1e-15.
+//
+// The fourth-order operator (1, -16; 60) / (12 h^2) takes no fixed point: there FP64 rounds
+// every product with 1 / 12 h^2 from the first step on, and an exact residual moves the
+// residual history of a solve by up to 3e-9 of its start (measured at 4097^2), through the
+// FP32 roundings of the inner cycle.
+//
+// With homogeneous data boundary values are 0 (not read); with data g they are read. A tile
+// with an infinity, a NaN, or only tiny values (E < 128) goes through the FP64 rows instead.
+#pragma once
+
+#include "device.cuh"
+
+namespace nsmg {
+namespace {
+
+constexpr int kFxW = 64, kFxH = 32;  // tile; kernels use 32 x 8 threads
+constexpr int kFxRW = kFxW + 2, kFxRH = kFxH + 2;  // with its halo
+constexpr int kFxRegion = kFxRW * kFxRH, kFxPer = (kFxRegion + 255) / 256;
+constexpr int kFxS0 = 6;  // fraction bits below the largest value's last one
+
+// x in units of 2^(E - 1075 - kFxS0), rounded to nearest; E >= exponent of x, E >= 128 (zeros
+// and subnormals come out as 0: they are shifted by E at least).
+__device__ __forceinline__ int64_t to_fixed(double x, int E) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int k = min(E - (int)((hi >> 20) & 0x7ffu), 63);
+  const uint64_t m = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << (kFxS0 + 1);
+  const int64_t q = (int64_t)(((m >> k) + 1) >> 1), neg = (int64_t)((int32_t)hi >> 31);
+  return (q ^ neg) - neg;
+}
+
+// (double)T for |T| <= 2^53, without the FP64 unit.
+__device__ __forceinline__ double narrow_to_double(int64_t T) {
+  const uint64_t neg = (uint64_t)(T >> 63), a = ((uint64_t)T ^ neg) - neg;
+  const int z = __clzll((long long)a);  // 10 .. 64
+  const uint64_t m = z < 11 ? a >> 1 : a << (z - 11);  // leading bit at 52 (2^53 itself is even)
+  const uint32_t hi = (uint32_t)(m >> 32) + ((uint32_t)(1085 - z) << 20);  // exponent 1086 - z, less the leading bit
+  return __hiloint2double((int)(a == 0 ? 0u : hi | ((uint32_t)neg & 0x80000000u)), (int)(uint32_t)m);
+}
+
+__device__ __forceinline__ void copy_async8(void* dst, const void* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(ok ? 8 : 0)
+               : "memory");
+}
+
+// Conversions off the common path. Calls, because the compiler would otherwise run them
+// under a predicate for every node, and a predicated FP64 instruction occupies the unit too
+// (8193^2, order 2: 796 us with them inlined, 709 without, before the copies ran ahead).
+__device__ __noinline__ double wide_to_double(int64_t T) { return (double)T; }
+__device__ __noinline__ float edge_to_float(double r, double scale) { return (float)(r * scale); }
+
+// fl32(r * 2^k).
+__device__ __forceinline__ float scaled_float(double r, int k, double scale) {
+  const uint32_t hi = (uint32_t)__double2hiint(r), lo = (uint32_t)__double2loint(r);
+  const int e = (int)((hi >> 20) & 0x7ff) - 896 + k;  // biased exponent of the float
+  if (e < 1 || e > 253) return edge_to_float(r, scale);  // 0, underflow, overflow, NaN
+  const uint32_t m = (hi & 0xfffffu) << 3 | lo >> 29, rem = lo & 0x1fffffffu;
+  const uint32_t up = rem > 0x10000000u - (m & 1u) ? 1u : 0u;  // half to even
+  return __uint_as_float((hi & 0x80000000u) | (((uint32_t)e << 23 | m) + up));
+}
+
+struct FxSmem {
+  int64_t q[2][kFxRegion];  // u, then its fixed-point values, of this tile and the next
+  uint32_t red[2][8];
+};
+
+// Copies u of the region of tile (i0, j0) to `dst` asynchronously, boundary values (unless
+// data) and what lies beyond as 0. Thread tid takes elements tid + 256 k.
+__device__ __forceinline__ void fx_fetch(const LevelGeo<double>& L, const double* __restrict__ u, int i0, int j0,
+                                         int64_t* dst) {
+  const int tid = threadIdx.y * kBX + threadIdx.x, lo = L.bdata ? 0 : 1, hi = L.bdata ? L.n : L.n - 1;
+  int x = tid % kFxRW, y = tid / kFxRW;
+#pragma unroll
+  for (int k = 0; k < kFxPer; ++k) {
+    if (tid + 256 * k >= kFxRegion) break;
+    const int i = i0 - 1 + x, j = j0 - 1 + y;
+    const bool ok = i >= lo && i <= hi && j >= lo && j <= hi;
+    copy_async8(dst + tid + 256 * k, ok ? u + (int64_t)j * L.pitch + i : u, ok);
+    x += 256 % kFxRW;
+    y += 256 / kFxRW;
+    if (x >= kFxRW) {
+      x -= kFxRW;
+      ++y;
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// One tile whose region fx_fetch has put into `buf` (its copies waited for by each thread):
+// store(i, j, r) for every unknown of columns i0 .. i0 + 63, rows j0 .. j0 + 31, in each
+// thread for its own nodes. 256 threads as (32, 8), all of them; the caller puts a barrier
+// before `buf` or sm.red is written again.
+template <bool EXACT, class Store>
+__device__ __forceinline__ void fx_tile(const LevelGeo<double>& L, const LevelDev<double>& LD, const double* __restrict__ u,
+                                        const double* __restrict__ f, int i0, int j0, int64_t* buf, FxSmem& sm,
+                                        Store store) {
+  constexpr int W = kFxRW, kRows = kFxH / 4;
+  const int tid = threadIdx.y * kBX + threadIdx.x, n = L.n;
+  const int cx = tid & 63, r0 = (tid >> 6) * kRows, i = i0 + cx;
+  double fv[kRows];
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) {
+    const int j = j0 + r0 + r;
+    fv[r] = i >= 1 && i < n && j < n ? f[(int64_t)j * L.pitch + i] : 0.0;
+  }
+  uint32_t mx = 0, any = 0;
+#pragma unroll
+  for (int k = 0; k < kFxPer; ++k) {
+    if (tid + 256 * k >= kFxRegion) break;
+    const uint64_t v = (uint64_t)buf[tid + 256 * k];
+    const uint32_t h = (uint32_t)(v >> 32) & 0x7fffffffu;
+    mx = max(mx, h);
+    any |= h | (uint32_t)v;
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  any = __reduce_or_sync(0xffffffffu, any);
+  if (threadIdx.x == 0) {
+    sm.red[0][threadIdx.y] = mx;
+    sm.red[1][threadIdx.y] = any;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    mx = max(mx, sm.red[0][k]);
+    any |= sm.red[1][k];
+  }
+  const int E = (int)(mx >> 20);
+  if (any != 0 && (E == 0x7ff || E < 128)) {  // uniform over the block
+    for (int r = 0; r < kRows; ++r) {
+      const int j = j0 + r0 + r;
+      if (i < 1 || i >= n || j < 1 || j >= n) continue;
+      const int64_t at = (int64_t)j * L.pitch + i;
+      store(i, j, Arith<double>::sub(f[at], apply_at<double, EXACT, 1>(LD, u, i, j, at, nullptr)));
+    }
+    return;
+  }
+  if (any != 0) {
+#pragma unroll
+    for (int k = 0; k < kFxPer; ++k) {
+      if (tid + 256 * k >= kFxRegion) break;
+      buf[tid + 256 * k] = to_fixed(__longlong_as_double(buf[tid + 256 * k]), E);
+    }
+  }
+  __syncthreads();
+  if (i < 1 || i >= n) return;
+  // L u = c0 T, T in units of 2^(E - 1075 - kFxS0) (any != 0: E >= 128, so the factor is
+  // normal; any == 0: the region holds zeros)
+  const double unit = any != 0 ? -L.c0 * __hiloint2double((E - 52 - kFxS0) << 20, 0) : 0.0;
+  const int64_t* q = buf + (r0 + 1) * W + cx + 1;
+  int64_t below = q[-W], here = q[0];
+#pragma unroll
+  for (int r = 0; r < kRows; ++r, q += W) {
+    const int64_t above = q[W], T = (below + q[-1] + q[1] + above) - (here << 2);  // |T| < 2^62
+    const int j = j0 + r0 + r;
+    if (j >= 1 && j < n) {
+      double t;
+      if ((uint64_t)(T + (1ll << 53)) <= (1ull << 54)) t = narrow_to_double(T);
+      else t = wide_to_double(T);
+      store(i, j, fma(unit, t, fv[r]));
+    }
+    below = here;
+    here = above;
+  }
+}
+
+}  // namespace
+}  // namespace nsmg

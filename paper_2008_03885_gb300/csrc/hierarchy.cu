@@ -876,11 +876,22 @@ std::vector<GroupRec<T>> group_records(const HostLevel& L, int32_t& maxg) {
   return out;
 }
 
+// Whether the level's operator is the cross c0 (1; -4) (LevelGeo::fx).
+int integer_cross(const HostLevel& L) {
+  if (L.shape.kind != kAxis || L.per || L.c.size() != 5 || !(L.c[0] < 0)) return 0;
+  const int dx[5] = {0, -1, 1, 0, 0}, dy[5] = {-1, 0, 0, 1, 0};
+  for (int k = 0; k < 5; ++k)
+    if (L.dxs[k] != dx[k] || L.dys[k] != dy[k] || L.c[k] != (k < 4 ? 1.0 : -4.0) * L.c[0]) return 0;
+  return 1;
+}
+
 // The level's descriptor and tables in one allocation, filled by one copy.
 template <typename T>
 mg_status upload_level(mg_handle* h, const HostLevel& L, LevelPair<T>& P, int bf16 = 0) {
   P.h = to_dev<T>(L);
   P.h.bf16 = bf16;
+  P.h.fx = integer_cross(L);
+  P.h.c0 = (T)L.c[0];
   const std::vector<GroupRec<T>> groups = group_records<T>(L, P.h.maxg);
   size_t bytes = 0;
   auto place = [&](size_t n) {
@@ -1851,8 +1862,9 @@ struct mg_batch {
   std::vector<BatchList<float>> lv32;
   std::vector<BatchLevel<double>> fin;  // finest FP64 levels (norms, refinement)
   BatchLevel<double>* d_fin = nullptr;
-  int* d_fin_prefix = nullptr;
-  int fin_tiles = 0;
+  int* d_fin_prefix = nullptr;   // rpt = 1 tiles
+  int* d_fin_prefix4 = nullptr;  // rpt = 4 tiles (mixed: refinement residual)
+  int fin_tiles = 0, fin_tiles4 = 0;
   std::vector<BatchLevel<double>> lv64_0;  // level-0 FP64 entries (u, f set per solve)
   int* d_active = nullptr;
   int* h_active = nullptr;
@@ -2155,9 +2167,15 @@ mg_status sync_create(mg_handle* const* handles, int count, mg_batch** out) {
     b->fin.push_back(e);
   }
   {
-    std::vector<int> pf(1, 0);
-    for (int p = 0; p < count; ++p) pf.push_back(pf.back() + batch_tiles(b->hs[p]->host[0].cols, b->hs[p]->host[0].rows, 1));
+    std::vector<int> pf(1, 0), pf4(1, 0);
+    for (int p = 0; p < count; ++p) {
+      const HostLevel& L = b->hs[p]->host[0];
+      pf.push_back(pf.back() + batch_tiles(L.cols, L.rows, 1));
+      pf4.push_back(pf4.back() + batch_tiles(L.cols, L.rows, 4));
+    }
     b->fin_tiles = pf.back();
+    b->fin_tiles4 = pf4.back();
+    if (b->mixed && (st = upload_vec(b, pf4, &b->d_fin_prefix4)) != MG_OK) return fail(st);
     if ((st = upload_vec(b, b->fin, &b->d_fin)) != MG_OK) return fail(st);
     if ((st = upload_vec(b, pf, &b->d_fin_prefix)) != MG_OK) return fail(st);
     if ((st = batch_alloc(b, (void**)&b->d_partial, std::max(b->fin_tiles, 1) * sizeof(double))) != MG_OK)
@@ -2228,8 +2246,8 @@ mg_status sync_solve(mg_batch* b, double* const* u, const double* const* f, doub
   CK(cudaMemcpyAsync(b->d_scale, b->h_scale, n * sizeof(double), cudaMemcpyHostToDevice, s));
   // ||f||^2 per problem
   b->launches += 2;
-  CK(launch_batch_norms(1, b->d_fin, b->d_fin_prefix, n, b->fin_tiles, b->d_active, b->d_scale, b->exact,
-                        b->d_partial, b->d_norm2, s));
+  CK(launch_batch_norms(1, b->d_fin, b->d_fin_prefix, n, b->fin_tiles, b->d_active, b->exact, b->d_partial,
+                        b->d_norm2, s));
   CK(cudaMemcpyAsync(b->h_norm2, b->d_norm2, n * sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   std::vector<double> fn2(b->h_norm2, b->h_norm2 + n), rr(n, 0.0);
@@ -2247,8 +2265,12 @@ mg_status sync_solve(mg_batch* b, double* const* u, const double* const* f, doub
   for (;;) {
     // residual norms (and, mixed, the scaled FP32 residual) of the active problems
     b->launches += 2;
-    CK(launch_batch_norms(b->mixed ? 0 : 2, b->d_fin, b->d_fin_prefix, n, b->fin_tiles, b->d_active, b->d_scale,
-                          b->exact, b->d_partial, b->d_norm2, s));
+    if (b->mixed)
+      CK(launch_batch_ir_residual(b->d_fin, b->d_fin_prefix4, n, b->fin_tiles4, b->d_active, b->d_scale, b->exact,
+                                  b->d_partial, b->d_norm2, s));
+    else
+      CK(launch_batch_norms(2, b->d_fin, b->d_fin_prefix, n, b->fin_tiles, b->d_active, b->exact, b->d_partial,
+                            b->d_norm2, s));
     CK(cudaMemcpyAsync(b->h_norm2, b->d_norm2, n * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     std::vector<double> next_scale(b->h_scale, b->h_scale + n);

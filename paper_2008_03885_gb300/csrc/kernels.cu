@@ -16,6 +16,7 @@
 #include "kernels.h"
 #include "device.cuh"
 #include "rows.cuh"
+#include "fixed.cuh"
 
 namespace nsmg {
 namespace {
@@ -1172,8 +1173,18 @@ __global__ void k_zero_boundary(int n, int pitch, T* __restrict__ u) {
   u[(int64_t)k * pitch + n] = T(0);        // i = n
 }
 
+// FP32 copy of a residual for the inner cycles: r scaled by 2^k, rounded once (to bfloat16
+// values in the storage trial).
+__device__ __forceinline__ float ir_value(double r, int k, double scale, int bf16) {
+  const float v = scaled_float(r, k, scale);
+  return bf16 ? __bfloat162float(__float2bfloat16_rn(v)) : v;
+}
+
 // Iterative-refinement residual: r = f - L u in FP64 (evaluation order of EXACT),
-// r32 = fl32(r * scale) for the FP32 inner cycles, and per-block sums of r^2.
+// r32 = fl32(r * scale) for the FP32 inner cycles, and per-block sums of r^2. Bound by the
+// FP64 units, so the scaling and rounding to FP32 are integer operations (scaled_float; the
+// multiply and the conversion took two of its 13 FP64 instructions a node: 4097^2, order 4,
+// 415 -> 330 us).
 //
 // With t32 (and L32, the FP32 level 0), the kernel also does the first half-sweep of the
 // FP32 cycle that follows from e = 0: red nodes get 0 + r32 omega / a_pp, black nodes 0.
@@ -1197,6 +1208,7 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<double>::value)
     dl[k] = L.delta[0][k];
   }
   const int pitch32 = L32.pitch;
+  const int k2 = (int)((__double2hiint(scale) >> 20) & 0x7ff) - 1023;  // scale = 2^k2
   double v = 0.0;
   for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
     const int ty = t / tiles_x;
@@ -1209,16 +1221,56 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<double>::value)
     const double s = (NT > 0 && fast_node(L, i, j)) ? apply_fast<double, EXACT, NA>(c, dl, u, at)
                                                     : apply_at<double, EXACT, 1>(L, u, i, j, at, nullptr);
     const double r = Arith<double>::sub(f[at], s);
-    const float r32v = (float)(r * scale);
-    const float rv = bf16 ? __bfloat162float(__float2bfloat16_rn(r32v)) : r32v;
+    const float rv = ir_value(r, k2, scale, bf16);
     const int64_t at32 = (int64_t)j * pitch32 + i;
     r32[at32] = rv;
-    v += r * r;
+    v = fma(r, r, v);
     if (t32) {
       float e = 0.f;
       if (is_red(L32, i, j) == 1) e = rnd(L32, relax_from_zero(rv, node_wd(L32, i, j)));
       t32[at32] = e;
     }
+  }
+  v = block_sum(v);
+  if (threadIdx.x == 0 && threadIdx.y == 0) partial[blockIdx.x] = v;
+}
+
+// The refinement residual in fixed point (fixed.cuh), the tiles in a flat order over one
+// resident wave as k_ir_residual's, the next tile's u in flight during the current one's
+// work (without: 709 us at 8193^2, order 2, with 3 blocks per SM; 502 with 4). FP64 rows
+// took 1208 us there; 200 us of HBM are its floor, integer issue and the waits between its
+// phases what bounds it.
+template <bool EXACT>
+__global__ void __launch_bounds__(kBX * kBY, 4)
+    k_ir_residual_fx(const __grid_constant__ LevelGeo<double> L, const LevelDev<double>* __restrict__ Lp,
+                     const double* __restrict__ u, const double* __restrict__ f, float* __restrict__ r32, double scale,
+                     double* __restrict__ partial, int tiles_x, int tiles, int bf16,
+                     const __grid_constant__ LevelGeo<float> L32, float* __restrict__ t32) {
+  __shared__ FxSmem sm;
+  const int k2 = (int)((__double2hiint(scale) >> 20) & 0x7ff) - 1023;
+  double v = 0.0;
+  auto fetch = [&](int t, int64_t* dst) {
+    const int ty = t / tiles_x, tx = t - ty * tiles_x;
+    fx_fetch(L, u, tx * kFxW, ty * kFxH, dst);
+  };
+  int which = 0;
+  if ((int)blockIdx.x < tiles) fetch(blockIdx.x, sm.q[0]);
+  for (int t = blockIdx.x; t < tiles; t += gridDim.x, which ^= 1) {
+    __syncthreads();  // the tile before is done with the other buffer
+    if (t + (int)gridDim.x < tiles) {
+      fetch(t + gridDim.x, sm.q[which ^ 1]);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    const int ty = t / tiles_x, tx = t - ty * tiles_x;
+    fx_tile<EXACT>(L, *Lp, u, f, tx * kFxW, ty * kFxH, sm.q[which], sm, [&](int i, int j, double r) {
+      const float rv = ir_value(r, k2, scale, bf16);
+      const int64_t at32 = (int64_t)j * L32.pitch + i;
+      r32[at32] = rv;
+      v = fma(r, r, v);
+      if (t32) t32[at32] = is_red(L32, i, j) == 1 ? rnd(L32, relax_from_zero(rv, node_wd(L32, i, j))) : 0.f;
+    });
   }
   v = block_sum(v);
   if (threadIdx.x == 0 && threadIdx.y == 0) partial[blockIdx.x] = v;
@@ -1446,8 +1498,7 @@ __global__ void __launch_bounds__(256) k_batch_coarsest_dense(const BatchLevel<T
 template <bool EXACT>
 __global__ void __launch_bounds__(kBX * kBY)
     k_batch_norm_partial(int mode, const BatchLevel<double>* __restrict__ E, const int* __restrict__ prefix, int ne,
-                         const int* __restrict__ active, const double* __restrict__ scale,
-                         double* __restrict__ partial) {
+                         const int* __restrict__ active, double* __restrict__ partial) {
   const int b = blockIdx.x;
   const int e = batch_entry(prefix, ne, b);
   const BatchLevel<double>& B = E[e];
@@ -1458,7 +1509,6 @@ __global__ void __launch_bounds__(kBX * kBY)
     const int bx = tile % B.tiles_x, by = tile / B.tiles_x;
     const int qb = bx * kBatchCols + 2 * threadIdx.x;
     const int j = by * kBY + threadIdx.y;
-    const double sc = scale[B.problem];
     for (int c = 0; c < 2; ++c) {
       const int q = qb + c;
       if (j >= L.rows || q >= L.cols) continue;
@@ -1467,11 +1517,49 @@ __global__ void __launch_bounds__(kBX * kBY)
       const int64_t at = (int64_t)j * L.pitch + q;
       if (mode != 1) {
         const double r = Arith<double>::sub(B.f[at], apply_at<double, EXACT>(L, B.u, i, j, at, nullptr));
-        if (mode == 0) B.r32[(int64_t)j * B.pitch32 + q] = (float)(r * sc);
         v += r * r;
       } else {
         v += B.f[at] * B.f[at];
       }
+    }
+  }
+  v = block_sum(v);
+  if (threadIdx.x == 0 && threadIdx.y == 0) partial[b] = v;
+}
+
+// Refinement residuals of a batch's finest levels: the 64 x 32 tiles and the arithmetic of
+// mg_solve's kernel for the level (k_ir_residual_fx, or k_ir_residual's rows), so that a
+// problem's FP32 right-hand side has the same bits in a batch as alone.
+template <bool EXACT>
+__global__ void __launch_bounds__(kBX * kBY, 4)
+    k_batch_ir_residual(const BatchLevel<double>* __restrict__ E, const int* __restrict__ prefix, int ne,
+                        const int* __restrict__ active, const double* __restrict__ scale, double* __restrict__ partial) {
+  __shared__ FxSmem sm;
+  const int b = blockIdx.x;
+  const int e = batch_entry(prefix, ne, b);
+  const BatchLevel<double>& B = E[e];
+  double v = 0.0;
+  if (active[B.problem]) {
+    const LevelDev<double>& L = *B.L;
+    const int tile = b - prefix[e], by = tile / B.tiles_x, bx = tile - by * B.tiles_x;
+    const double sc = scale[B.problem];
+    const int k2 = (int)((__double2hiint(sc) >> 20) & 0x7ff) - 1023;
+    auto store = [&](int i, int j, double r) {
+      B.r32[(int64_t)j * B.pitch32 + i] = scaled_float(r, k2, sc);
+      v = fma(r, r, v);
+    };
+    if (L.fx) {
+      fx_fetch(L, B.u, bx * kFxW, by * kFxH, sm.q[0]);
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      fx_tile<EXACT>(L, L, B.u, B.f, bx * kFxW, by * kFxH, sm.q[0], sm, store);
+    } else {
+      for (int r = 0; r < kFxH / kBY; ++r)
+        for (int c = 0; c < 2; ++c) {
+          const int i = bx * kFxW + 2 * threadIdx.x + c, j = by * kFxH + r * kBY + threadIdx.y;
+          if (!interior(L, i, j)) continue;
+          const int64_t at = (int64_t)j * L.pitch + i;
+          store(i, j, Arith<double>::sub(B.f[at], apply_at<double, EXACT>(L, B.u, i, j, at, nullptr)));
+        }
     }
   }
   v = block_sum(v);
@@ -2165,9 +2253,24 @@ cudaError_t launch_ir_residual_as(const LevelPair<double>& L, const double* u, c
   return cudaGetLastError();
 }
 
+template <bool EXACT>
+cudaError_t launch_ir_residual_fx(const LevelPair<double>& L, const double* u, const double* f,
+                                  const LevelPair<float>& L32, float* r32, double scale, double* partial, double* out,
+                                  cudaStream_t s, int bf16, float* t32) {
+  const int tx = (L.h.cols + kFxW - 1) / kFxW, tiles = tx * ((L.h.rows + kFxH - 1) / kFxH);
+  const int blocks = std::min({tiles, kMaxPartials, resident_blocks<k_ir_residual_fx<EXACT>>()});
+  k_ir_residual_fx<EXACT><<<blocks, dim3(kBX, kBY), 0, s>>>(L.h, L.d, u, f, r32, scale, partial, tx, tiles, bf16,
+                                                                L32.h, t32);
+  k_sum_partials<<<1, dim3(kBX, kBY), 0, s>>>(partial, blocks, out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_ir_residual(const LevelPair<double>& L, bool exact, const double* u, const double* f,
                                const LevelPair<float>& L32, float* r32, double scale, double* partial,
                                double* out, cudaStream_t s, int bf16, float* t32) {
+  if (L.h.fx)
+    return exact ? launch_ir_residual_fx<true>(L, u, f, L32, r32, scale, partial, out, s, bf16, t32)
+                 : launch_ir_residual_fx<false>(L, u, f, L32, r32, scale, partial, out, s, bf16, t32);
   const int ntf = fast_nt(L.h);
   if (ntf == 9)
     return exact ? launch_ir_residual_as<true, 9>(L, u, f, L32, r32, scale, partial, out, s, bf16, t32)
@@ -2266,11 +2369,21 @@ cudaError_t launch_batch_step(int op, const BatchLevel<T>* entries, const int* p
 }
 
 cudaError_t launch_batch_norms(int mode, const BatchLevel<double>* entries, const int* prefix, int ne,
-                               int total_tiles, const int* active, const double* scale, bool exact,
-                               double* partial, double* norm2, cudaStream_t s) {
+                               int total_tiles, const int* active, bool exact, double* partial, double* norm2,
+                               cudaStream_t s) {
   if (ne <= 0 || total_tiles <= 0) return cudaSuccess;
-  if (exact) k_batch_norm_partial<true><<<total_tiles, dim3(kBX, kBY), 0, s>>>(mode, entries, prefix, ne, active, scale, partial);
-  else k_batch_norm_partial<false><<<total_tiles, dim3(kBX, kBY), 0, s>>>(mode, entries, prefix, ne, active, scale, partial);
+  if (exact) k_batch_norm_partial<true><<<total_tiles, dim3(kBX, kBY), 0, s>>>(mode, entries, prefix, ne, active, partial);
+  else k_batch_norm_partial<false><<<total_tiles, dim3(kBX, kBY), 0, s>>>(mode, entries, prefix, ne, active, partial);
+  k_batch_norm_sum<<<ne, dim3(kBX, kBY), 0, s>>>(entries, prefix, active, partial, norm2);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_ir_residual(const BatchLevel<double>* entries, const int* prefix, int ne, int total_tiles,
+                                     const int* active, const double* scale, bool exact, double* partial,
+                                     double* norm2, cudaStream_t s) {
+  if (ne <= 0 || total_tiles <= 0) return cudaSuccess;
+  if (exact) k_batch_ir_residual<true><<<total_tiles, dim3(kBX, kBY), 0, s>>>(entries, prefix, ne, active, scale, partial);
+  else k_batch_ir_residual<false><<<total_tiles, dim3(kBX, kBY), 0, s>>>(entries, prefix, ne, active, scale, partial);
   k_batch_norm_sum<<<ne, dim3(kBX, kBY), 0, s>>>(entries, prefix, active, partial, norm2);
   return cudaGetLastError();
 }

@@ -192,12 +192,16 @@ inline int batch_tiles(int cols, int rows, int rpt) {
 template <typename T>
 cudaError_t launch_batch_step(int op, const BatchLevel<T>* entries, const int* prefix, int ne, int total_tiles,
                               int rpt, const int* active, bool exact, cudaStream_t s);
-// Finest levels of a batch (FP64 entries, rpt = 1 tiles). mode 0: r = f - L u,
-// r32 = fl32(r * scale[problem]) and partial[tile] = sum of r^2; mode 1: partial =
-// sum of f^2; mode 2: partial = sum of r^2 only. Then norm2[problem] = the entry's partials added in a fixed order.
+// Finest levels of a batch (FP64 entries, rpt = 1 tiles). mode 1: partial[tile] = sum of
+// f^2; mode 2: sum of (f - L u)^2. Then norm2[problem] = the entry's partials added in a
+// fixed order.
 cudaError_t launch_batch_norms(int mode, const BatchLevel<double>* entries, const int* prefix, int ne,
-                               int total_tiles, const int* active, const double* scale, bool exact,
-                               double* partial, double* norm2, cudaStream_t s);
+                               int total_tiles, const int* active, bool exact, double* partial, double* norm2,
+                               cudaStream_t s);
+// r = f - L u, r32 = fl32(r * scale[problem]) and norm2[problem] = sum of r^2 (rpt = 4 tiles).
+cudaError_t launch_batch_ir_residual(const BatchLevel<double>* entries, const int* prefix, int ne, int total_tiles,
+                                     const int* active, const double* scale, bool exact, double* partial,
+                                     double* norm2, cudaStream_t s);
 // u += e32 / scale[problem] on the finest levels.
 cudaError_t launch_batch_ir_update(const BatchLevel<double>* entries, const int* prefix, int ne, int total_tiles,
                                    const int* active, const double* scale, cudaStream_t s);
