@@ -891,6 +891,12 @@ mg_status upload_level(mg_handle* h, const HostLevel& L, LevelPair<T>& P, int bf
   P.h = to_dev<T>(L);
   P.h.bf16 = bf16;
   P.h.fx = integer_cross(L);
+  P.h.pow2 = L.c.size() == 5 || L.c.size() == 9 ? 1 : 0;
+  for (size_t k = 0; k + 1 < L.c.size(); ++k) {
+    int e;
+    const double m = std::frexp(std::fabs(L.c[k]), &e);
+    if (m != 0.5 || e < 1 || e > 201) P.h.pow2 = 0;
+  }
   P.h.c0 = (T)L.c[0];
   const std::vector<GroupRec<T>> groups = group_records<T>(L, P.h.maxg);
   size_t bytes = 0;

@@ -84,6 +84,7 @@ struct LevelGeo {
   int32_t fxe, fye;  // last fast-node i and j: n - per - rx, n - per - ry
   int32_t bdata;     // level 0 with Dirichlet data g: fast rows read the boundary entries,
                      // which class rows drop
+  int32_t pow2;      // 1: 5 or 9 terms, the coefficients before the last powers of two in [1, 2^200]
   int32_t fx;        // 1: an axis level with Dirichlet boundaries and the 5-point cross c0 (1; -4)
   T c0;              // c[0]
 };
