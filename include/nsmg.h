@@ -290,7 +290,7 @@ mg_status mg_level_prolong_add(mg_handle* h, int level, double* u_fine, const do
    `workers` internal non-blocking streams, each driven by a host thread that takes the
    next unsolved problem, largest first. Meanwhile the calling thread runs the
    level-synchronous schedule of the other problems. A large problem's own mg_solve
-   runs its single-problem kernels (TMA tiles, fused coarse tail); a small problem's
+   runs its single-problem kernels (TMA tiles); a small problem's
    levels leave most SMs idle alone, which the level-synchronous steps fill. The
    caller's stream waits for all of it. Results stay bitwise those of mg_solve alone.
    mg_batch_options (opt may be NULL: the defaults):
