@@ -81,16 +81,19 @@ struct FxSmem {
 };
 
 // Copies u of the region of tile (i0, j0) to `dst` asynchronously, boundary values (unless
-// data) and what lies beyond as 0. Thread tid takes elements tid + 256 k.
+// data) and what lies beyond as 0; the grid's corners too, which no row reads: whatever a
+// caller's array holds there must not set the tile's scale. Thread tid takes elements
+// tid + 256 k.
 __device__ __forceinline__ void fx_fetch(const LevelGeo<double>& L, const double* __restrict__ u, int i0, int j0,
                                          int64_t* dst) {
-  const int tid = threadIdx.y * kBX + threadIdx.x, lo = L.bdata ? 0 : 1, hi = L.bdata ? L.n : L.n - 1;
+  const int tid = threadIdx.y * kBX + threadIdx.x, n = L.n;
   int x = tid % kFxRW, y = tid / kFxRW;
 #pragma unroll
   for (int k = 0; k < kFxPer; ++k) {
     if (tid + 256 * k >= kFxRegion) break;
     const int i = i0 - 1 + x, j = j0 - 1 + y;
-    const bool ok = i >= lo && i <= hi && j >= lo && j <= hi;
+    const bool in_i = i >= 1 && i < n, in_j = j >= 1 && j < n;
+    const bool ok = (in_i && in_j) || (L.bdata && ((in_i && (j == 0 || j == n)) || (in_j && (i == 0 || i == n))));
     copy_async8(dst + tid + 256 * k, ok ? u + (int64_t)j * L.pitch + i : u, ok);
     x += 256 % kFxRW;
     y += 256 / kFxRW;
