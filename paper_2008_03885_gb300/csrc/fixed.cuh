@@ -9,11 +9,12 @@
 // and r = f - s T is one fused multiply-add; FP64 keeps two operations a node (that one and
 // the square for the norm).
 //
-// Precision. A value of exponent E or up to 6 below is exact; smaller ones are rounded to
-// half a unit, 2^-7 of the largest value's last bit, where FP64 rounds every partial sum (up
-// to 8 times the value) to half its own last bit. Mixed solves run to their floor keep a
-// relative residual of 0.45-0.5 of the FP64 sum's (8193^2: 9.3e-14 for 2.0e-13), and their
-// error against the exact discrete solution falls from 1e-14-3e-13 to 5e-16-1e-15.
+// Precision. A node takes the integer sum only if each of its five values has no bit below
+// the unit (all values within 6 binades of the largest do): T is then exact, r has the
+// rounding of T to 53 bits and of the fused multiply-add, and is nowhere further off than the
+// FP64 row, which rounds its partial sums too. A value that loses bits is made odd (the
+// format's last bit is kept for that), and the nodes that read one take their FP64 row: beside
+// zeros of u, in the corners of the grid, in tiles of wide range.
 //
 // The fourth-order operator (1, -16; 60) / (12 h^2) takes no fixed point: there FP64 rounds
 // every product with 1 / 12 h^2 from the first step on, and an exact residual moves the
@@ -23,6 +24,8 @@
 // With homogeneous data boundary values are 0 (not read); with data g they are read. A tile
 // with an infinity, a NaN, or only tiny values (E < 128) goes through the FP64 rows instead.
 #pragma once
+
+#include <type_traits>
 
 #include "device.cuh"
 
@@ -34,14 +37,17 @@ constexpr int kFxRW = kFxW + 2, kFxRH = kFxH + 2;  // with its halo
 constexpr int kFxRegion = kFxRW * kFxRH, kFxPer = (kFxRegion + 255) / 256;
 constexpr int kFxS0 = 6;  // fraction bits below the largest value's last one
 
-// x in units of 2^(E - 1075 - kFxS0), rounded to nearest; E >= exponent of x, E >= 128 (zeros
-// and subnormals come out as 0: they are shifted by E at least).
+// x in units of 2^(E - 1075 - kFxS0 - 1): even if exact in units twice that (values of exponent
+// E - kFxS0 and above, and 0), odd if not (MARK; else not told); E >= exponent of x, E >= 128.
+template <bool MARK>
 __device__ __forceinline__ int64_t to_fixed(double x, int E) {
   const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
   const int k = min(E - (int)((hi >> 20) & 0x7ffu), 63);
   const uint64_t m = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << (kFxS0 + 1);
-  const int64_t q = (int64_t)(((m >> k) + 1) >> 1), neg = (int64_t)((int32_t)hi >> 31);
-  return (q ^ neg) - neg;
+  uint64_t q = m >> k;  // 0 for zeros and subnormals: k = 63
+  if (MARK && k > kFxS0 + 1 && (hi << 1 | lo) != 0) q |= (m << (64 - k)) != 0 ? 1u : 0u;
+  const int64_t neg = (int64_t)((int32_t)hi >> 31);
+  return ((int64_t)q ^ neg) - neg;
 }
 
 // (double)T for |T| <= 2^53, without the FP64 unit.
@@ -77,7 +83,7 @@ __device__ __forceinline__ float scaled_float(double r, int k, double scale) {
 
 struct FxSmem {
   int64_t q[2][kFxRegion];  // u, then its fixed-point values, of this tile and the next
-  uint32_t red[2][8];
+  uint32_t red[3][8];
 };
 
 // Copies u of the region of tile (i0, j0) to `dst` asynchronously, boundary values (unless
@@ -122,63 +128,89 @@ __device__ __forceinline__ void fx_tile(const LevelGeo<double>& L, const LevelDe
     const int j = j0 + r0 + r;
     fv[r] = i >= 1 && i < n && j < n ? f[(int64_t)j * L.pitch + i] : 0.0;
   }
-  uint32_t mx = 0, any = 0;
+  // largest high word, smallest one less 1 (zeros, and values below 2^-1042, which reach neither
+  // the FP32 residual nor the norm, wrap to the largest), any bit
+  uint32_t mx = 0, mn = ~0u, any = 0;
 #pragma unroll
   for (int k = 0; k < kFxPer; ++k) {
     if (tid + 256 * k >= kFxRegion) break;
     const uint64_t v = (uint64_t)buf[tid + 256 * k];
     const uint32_t h = (uint32_t)(v >> 32) & 0x7fffffffu;
     mx = max(mx, h);
+    mn = min(mn, h - 1);
     any |= h | (uint32_t)v;
   }
   mx = __reduce_max_sync(0xffffffffu, mx);
+  mn = __reduce_min_sync(0xffffffffu, mn);
   any = __reduce_or_sync(0xffffffffu, any);
   if (threadIdx.x == 0) {
     sm.red[0][threadIdx.y] = mx;
     sm.red[1][threadIdx.y] = any;
+    sm.red[2][threadIdx.y] = mn;
   }
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     mx = max(mx, sm.red[0][k]);
     any |= sm.red[1][k];
+    mn = min(mn, sm.red[2][k]);
   }
   const int E = (int)(mx >> 20);
+  uint32_t rest = 0;  // bit r: the node of row r takes its FP64 row
   if (any != 0 && (E == 0x7ff || E < 128)) {  // uniform over the block
-    for (int r = 0; r < kRows; ++r) {
-      const int j = j0 + r0 + r;
-      if (i < 1 || i >= n || j < 1 || j >= n) continue;
-      const int64_t at = (int64_t)j * L.pitch + i;
-      store(i, j, Arith<double>::sub(f[at], apply_at<double, EXACT, 1>(LD, u, i, j, at, nullptr)));
-    }
-    return;
-  }
-  if (any != 0) {
+    rest = (1u << kRows) - 1;
+  } else {
+    // whether some value may lose bits (uniform over the block)
+    const bool marks = (int)((mx >> 20) - ((mn + 1) >> 20)) > kFxS0 && mn != ~0u;
+    auto convert = [&](auto mark) {
 #pragma unroll
-    for (int k = 0; k < kFxPer; ++k) {
-      if (tid + 256 * k >= kFxRegion) break;
-      buf[tid + 256 * k] = to_fixed(__longlong_as_double(buf[tid + 256 * k]), E);
+      for (int k = 0; k < kFxPer; ++k) {
+        if (tid + 256 * k >= kFxRegion) break;
+        buf[tid + 256 * k] = to_fixed<decltype(mark)::value>(__longlong_as_double(buf[tid + 256 * k]), E);
+      }
+    };
+    if (any != 0) {
+      if (marks) convert(std::true_type());
+      else convert(std::false_type());
+    }
+    __syncthreads();
+    // L u = c0 T, T in units of 2^(E - 1075 - kFxS0 - 1) (any != 0: E >= 128, so the factor is
+    // normal; any == 0: the region holds zeros)
+    const double unit = any != 0 ? -L.c0 * __hiloint2double((E - 53 - kFxS0) << 20, 0) : 0.0;
+    // Most tiles need no marks and run without the tests: 8193^2, order 2, solved u: 554 us
+    // (595 with marks in every tile, 515 with none at all, bits lost; white noise, where most
+    // warps hold a marked row, 1005; FP64 rows 1208)
+    auto walk = [&](auto marked) {
+      const int64_t* q = buf + (r0 + 1) * W + cx + 1;
+      int64_t below = q[-W], here = q[0];
+#pragma unroll
+      for (int r = 0; r < kRows; ++r, q += W) {
+        const int64_t above = q[W], left = q[-1], right = q[1], T = (below + left + right + above) - (here << 2);
+        const int j = j0 + r0 + r;
+        if (decltype(marked)::value &&
+            (((uint32_t)below | (uint32_t)left | (uint32_t)right | (uint32_t)above | (uint32_t)here) & 1u)) {
+          rest |= 1u << r;
+        } else if (j >= 1 && j < n) {  // |T| < 2^63
+          double t;
+          if ((uint64_t)(T + (1ll << 53)) <= (1ull << 54)) t = narrow_to_double(T);
+          else t = wide_to_double(T);
+          store(i, j, fma(unit, t, fv[r]));
+        }
+        below = here;
+        here = above;
+      }
+    };
+    if (i >= 1 && i < n) {
+      if (marks) walk(std::true_type());
+      else walk(std::false_type());
     }
   }
-  __syncthreads();
-  if (i < 1 || i >= n) return;
-  // L u = c0 T, T in units of 2^(E - 1075 - kFxS0) (any != 0: E >= 128, so the factor is
-  // normal; any == 0: the region holds zeros)
-  const double unit = any != 0 ? -L.c0 * __hiloint2double((E - 52 - kFxS0) << 20, 0) : 0.0;
-  const int64_t* q = buf + (r0 + 1) * W + cx + 1;
-  int64_t below = q[-W], here = q[0];
-#pragma unroll
-  for (int r = 0; r < kRows; ++r, q += W) {
-    const int64_t above = q[W], T = (below + q[-1] + q[1] + above) - (here << 2);  // |T| < 2^62
-    const int j = j0 + r0 + r;
-    if (j >= 1 && j < n) {
-      double t;
-      if ((uint64_t)(T + (1ll << 53)) <= (1ull << 54)) t = narrow_to_double(T);
-      else t = wide_to_double(T);
-      store(i, j, fma(unit, t, fv[r]));
-    }
-    below = here;
-    here = above;
+  // one pass for the marked rows of all lanes, whichever rows they are
+  for (; rest; rest &= rest - 1) {
+    const int j = j0 + r0 + __ffs((int)rest) - 1;
+    if (i < 1 || i >= n || j < 1 || j >= n) continue;
+    const int64_t at = (int64_t)j * L.pitch + i;
+    store(i, j, Arith<double>::sub(f[at], apply_at<double, EXACT, 1>(LD, u, i, j, at, nullptr)));
   }
 }
 
