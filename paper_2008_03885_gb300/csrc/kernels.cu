@@ -1612,11 +1612,13 @@ __global__ void __launch_bounds__(kBX * kBY)
 // ---- shared-memory-resident tail ---------------------------------------------
 // The levels from sm_top down live in one block's shared memory, each in its storage
 // layout, and the block runs their whole sub-cycle with a barrier between phases. Class
-// rows are evaluated by octets of lanes in FP64 and by one thread a node in FP32 (rows.cuh;
-// with the values in shared memory and the records in L1 the octets' chain of shuffles is
-// the longer one); arithmetic per node is the same as relax_value / apply_at /
-// restrict_value / prolong_value. Measured, three W cycles of 256^2, order 4: FP64 1197 ->
-// 782 ms, mixed 485 -> 403 ms (548 with octets) against one thread per storage element.
+// rows are evaluated by octets of lanes in FP64 with the exact order, and by one thread a
+// node in FP32 and with FMA (rows.cuh; with the values in shared memory and the records in L1
+// the octets' chain of shuffles is the longer one, and with FMA they pass the sum from lane
+// to lane term by term); arithmetic per node is the same as relax_value / apply_at /
+// restrict_value / prolong_value. Measured against one thread per storage element, order 4:
+// three W cycles of 256^2, FP64 1197 -> 782 ms, mixed 485 -> 403 ms (548 with octets); one W
+// cycle of 64^2, FP64 with FMA, 15.9 -> 13.1 ms (26.2 with octets).
 //
 // A sweep reads the level's current array A and writes the other one, B: the red phase
 // reads A and writes B's red nodes, the black phase reads B at red and A at black nodes
@@ -1630,8 +1632,10 @@ __global__ void __launch_bounds__(kBX * kBY)
 // a warp): a lone octet is the shorter chain, but past about two octet warps to each FP64
 // unit (FP32: issue slots) the threads' 60 FP64 instructions for 32 nodes beat 20 for four.
 constexpr int kTailSmemThreads = 512;
-template <typename T>
-constexpr int kTailThreadNodes = sizeof(T) == 8 ? 32 : 16;
+template <typename T, bool EXACT>
+constexpr bool kTailOctets = sizeof(T) == 8 && EXACT;  // class rows by octets
+template <typename T, bool EXACT>
+constexpr int kTailThreadNodes = kTailOctets<T, EXACT> ? 32 : 16;
 constexpr int kTailStencil = 48;  // longest interior stencil evaluated by threads (others: octets)
 
 template <typename T>
@@ -1652,12 +1656,12 @@ struct TailPhase {
   uint32_t m;  // slot / w = slot m >> 32 (w = 1: m = 0)
 };
 
-template <typename T>
+template <typename T, bool EXACT>
 __device__ __forceinline__ TailPhase tail_phase(const LevelGeo<T>& L, int c) {
   TailPhase P;
   const int rot = L.kind == kRot;
   const int nodes = (L.n - L.lo) * (L.n - L.lo) / ((rot ? 2 : 1) * (c == kAllNodes ? 1 : 2));
-  P.S = make_strips(L, c, nodes <= kTailThreadNodes<T> || L.nt > kTailStencil);
+  P.S = make_strips(L, c, nodes <= kTailThreadNodes<T, EXACT> || L.nt > kTailStencil);
   P.first = P.S.rstep == 2 ? L.ry + ((L.ry ^ c) & 1) : L.ry;
   P.w = P.S.all ? 0 : (L.fxe - L.rx) / P.S.cstep + 1;
   P.total = P.S.all || P.first > L.fye ? 0 : ((L.fye - P.first) / P.S.rstep + 1) * P.w;
@@ -1696,7 +1700,7 @@ __global__ void __launch_bounds__(kTailSmemThreads, 1)
     }
   }
   __syncthreads();
-  for (int x = tid; x < 3 * nst; x += kTailSmemThreads) phase[top + x / 3][x % 3] = tail_phase(geo[top + x / 3], x % 3);
+  for (int x = tid; x < 3 * nst; x += kTailSmemThreads) phase[top + x / 3][x % 3] = tail_phase<T, EXACT>(geo[top + x / 3], x % 3);
   {  // top level: f, and u unless it is zero, from global memory
     const LevelGeo<T>& L = geo[top];
     for (int k = tid; k < L.rows * L.pitch; k += kTailSmemThreads) {
@@ -1717,7 +1721,7 @@ __global__ void __launch_bounds__(kTailSmemThreads, 1)
     const int rot = L.kind == kRot;
     const TailPhase& P = phase[l][c];
     const StripGeo& S = P.S;
-    constexpr int kPer = sizeof(T) == 8 ? 4 : 32;  // class nodes to a chunk
+    constexpr int kPer = kTailOctets<T, EXACT> ? 4 : 32;  // class nodes to a chunk
     const int oc = (S.total + kPer - 1) / kPer, chunks = oc + (P.total + 31) / 32;
     auto val = [&](int k, T v, T wd) {
       const T r = Arith<T>::sub(F[k], v);
