@@ -1345,22 +1345,24 @@ void emit_tail_smem(const mg_handle* h, int l, bool start, std::vector<int4>& pr
 // `max_unknowns` unknowns down to the coarsest to the tail kernel.
 // smem_elems > 0: instead of the unknowns threshold, take the first level (below the
 // finest) from which all levels' u, t and f fit in that many shared-memory elements,
-// and run the tail from shared memory.
+// and run the tail from shared memory. The tails store FP32 values as they are, so levels of
+// the bfloat16 storage trial stay out of them.
 template <typename T>
 mg_status build_tail(mg_handle* h, int64_t max_unknowns, int64_t smem_elems = 0) {
   Hier<T>& H = hier<T>(h);
   const int nl = (int)h->host.size();
+  const int first = sizeof(T) == 4 ? std::max(1, (int)h->opt.bf16_levels) : 1;
   int lt = -1;
   int64_t elems = 0;
   if (smem_elems > 0) {
-    for (int l = nl - 1; l >= 1; --l) {
+    for (int l = nl - 1; l >= first; --l) {
       const int64_t e = elems + 3 * (int64_t)h->host[l].rows * h->host[l].pitch;
       if (e > smem_elems) break;
       elems = e;
       if (l + 1 < nl) lt = l;
     }
   } else {
-    for (int l = 1; l + 1 < nl; ++l)
+    for (int l = first; l + 1 < nl; ++l)
       if (h->host[l].unknowns <= max_unknowns) { lt = l; break; }
   }
   if (lt < 0 || nl > kTailMaxLevels) return MG_OK;

@@ -73,3 +73,13 @@ def test_fp64_w_cycles_match_the_oracle(setting, smooth):
     u, hist, _ = solve(setting, smooth, gamma=2)
     assert np.array_equal(u[o.levels[0].pj, o.levels[0].pi], uo)
     assert np.max(np.abs(np.array(hist) - np.array(ho)) / np.array(ho)) <= 1e-12
+
+
+@pytest.mark.parametrize("tail", [dict(gamma=2), dict(gamma=2, tail_unknowns=300), dict(tail_unknowns=300)])
+@pytest.mark.parametrize("levels", [1, 3, 4])
+def test_levels_of_the_bfloat16_trial_are_not_in_a_tail(levels, tail):
+    """Every value stored on the finest k levels is rounded, whatever kernel runs the level."""
+    o = dict(precision=mg.MG_PREC_MIXED_FP32, bf16_levels=levels)
+    u, hist, _ = solve("dirichlet", "rb2", **o, **tail)
+    u2, hist2, _ = solve("dirichlet", "rb2", **o, **{**tail, "tail_unknowns": -1})
+    assert np.array_equal(u, u2) and hist == hist2
