@@ -140,8 +140,9 @@ typedef struct {
                           step cost more than extra steps) */
   int32_t tail_unknowns;/* > 0: levels (below the finest) with at most this many unknowns run in
                            one thread-block-cluster kernel; -1: never (every level as separate
-                           launches); 0 (default): W cycles run the levels that fit one block's
-                           shared memory in one kernel, other cycles have separate launches */
+                           launches); 0 (default): W cycles, Jacobi smoothing and sweep_kernel = 2
+                           run the levels that fit one block's shared memory in one kernel,
+                           other cycles have separate launches */
   int32_t tail_ctas;   /* CTAs of that cluster (1..16); 0 = largest the device schedules */
   int32_t sweep_kernel;/* red-black sweeps: 0 = auto (mixed precision: large FP32 axis levels with a
                           5- or 9-point cross stencil run TMA-staged shared-memory tile kernels,

@@ -1418,21 +1418,28 @@ mg_status build_tail(mg_handle* h, int64_t max_unknowns, int64_t smem_elems = 0)
   return MG_OK;
 }
 
-// The tail that the options ask for. V and Wn cycles by default have none: small levels as
-// separate launches with programmatic dependent launch are the fastest form (measured on
-// GB300, launches / their sub-cycle in one block's shared memory, best of five budgets:
-// FP64 128^2 1.88 / 1.94 ms, FP64 4096^2 38.4 / 38.6, mixed 4096^2 9.63 / 9.76; in a cluster
-// of 16 CTAs slower still, as a cluster barrier after stores into the other CTAs' shared
-// memory takes 0.65-1.5 us and an empty kernel in a graph 0.85 us). A W cycle visits level
-// l 2^l times, so there every level kept out of the launch list halves its length.
-// Budgets in values of u, t and f; three W cycles of 256^2, order 4: mixed 415 / 403 ms with
-// 3K / 6K, FP64 782 ms with 3K and 4.5K and 9-13% more with 7K and 13.5K.
-constexpr int64_t kTailSmemElemsFp32 = 6 * 1024, kTailSmemElemsFp64 = 4608;
+// The tail that the options ask for. V and Wn cycles with red-black half-sweeps by default
+// have none: small levels as separate launches, their class rows by octets and started early
+// (programmatic dependent launch), are the fastest form (measured on GB300, launches / their
+// sub-cycle in one block's shared memory, best of five budgets: FP64 128^2 1.88 / 1.94 ms, FP64
+// 4096^2 38.4 / 38.6, mixed 4096^2 9.63 / 9.76; in a cluster of 16 CTAs slower still, as a
+// cluster barrier after stores into the other CTAs' shared memory takes 0.65-1.5 us and an
+// empty kernel in a graph 0.85 us). Jacobi sweeps and the one-kernel red-black sweeps
+// (sweep_kernel = 2) have neither octets nor the early start, and keep the tail (us a cycle,
+// launches / tail, order 4: Jacobi V(2,1) mixed 32^2 290 / 136, 128^2 480 / 296, 512^2 678 /
+// 498, FP64 32^2 347 / 236; Jacobi Wn mixed 32^2 859 / 284; sweep_kernel = 2, mixed 512^2 1461 /
+// 1187). A W cycle visits level l 2^l times, so there every level kept out of the launch list
+// halves its length. Budgets in values of u, t and f, rows padded to 32: 10K holds the rotated
+// level of 32^2 and all below. FP32, us a cycle, 6K / 10K: Jacobi V mixed 128^2 359 / 296, W
+// mixed 64^2 8410 / 8133; FP64 three W cycles of 256^2: 782 ms with 3K and 4.5K and 9-13%
+// more with 7K and 13.5K.
+constexpr int64_t kTailSmemElemsFp32 = 10 * 1024, kTailSmemElemsFp64 = 4608;
 template <typename T>
 mg_status default_tail(mg_handle* h) {
   const mg_options& o = h->opt;
   if (o.tail_unknowns > 0) return build_tail<T>(h, o.tail_unknowns);
-  if (o.tail_unknowns < 0 || o.gamma != 2) return MG_OK;
+  const bool half_sweeps = o.smoother == MG_SMOOTH_REDBLACK && o.sweep_kernel != 2;
+  if (o.tail_unknowns < 0 || (o.gamma != 2 && half_sweeps)) return MG_OK;
   return build_tail<T>(h, 0, sizeof(T) == 8 ? kTailSmemElemsFp64 : kTailSmemElemsFp32);
 }
 

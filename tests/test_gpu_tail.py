@@ -83,3 +83,27 @@ def test_levels_of_the_bfloat16_trial_are_not_in_a_tail(levels, tail):
     u, hist, _ = solve("dirichlet", "rb2", **o, **tail)
     u2, hist2, _ = solve("dirichlet", "rb2", **o, **{**tail, "tail_unknowns": -1})
     assert np.array_equal(u, u2) and hist == hist2
+
+
+@pytest.mark.parametrize("precision", [mg.MG_PREC_FP64, mg.MG_PREC_MIXED_FP32])
+@pytest.mark.parametrize("fma", [0, 1])
+@pytest.mark.parametrize("gamma", [1, 3])
+@pytest.mark.parametrize("setting", ["dirichlet", "dense8", "standard", "periodic"])
+def test_v_cycles_with_jacobi_have_a_tail(setting, gamma, fma, precision):
+    """Jacobi levels are launches of one thread per class node; the small ones stay in the tail."""
+    o = dict(gamma=gamma, precision=precision, fma_contract=fma)
+    u, hist, launches = solve(setting, "jacobi", **o)
+    u2, hist2, launches2 = solve(setting, "jacobi", tail_unknowns=-1, **o)
+    assert np.array_equal(u, u2) and hist == hist2
+    assert launches < launches2
+
+
+@pytest.mark.parametrize("precision", [mg.MG_PREC_FP64, mg.MG_PREC_MIXED_FP32])
+@pytest.mark.parametrize("fma", [0, 1])
+@pytest.mark.parametrize("setting", ["dirichlet", "dense8", "standard"])
+def test_v_cycles_with_one_kernel_sweeps_have_a_tail(setting, fma, precision):
+    o = dict(precision=precision, fma_contract=fma, sweep_kernel=2)
+    u, hist, launches = solve(setting, "rb2", **o)
+    u2, hist2, launches2 = solve(setting, "rb2", tail_unknowns=-1, **o)
+    assert np.array_equal(u, u2) and hist == hist2
+    assert launches < launches2
