@@ -12,11 +12,15 @@
 // coefficient and up to eight offsets in 48 bytes; groups g and g + 8 of the row in lane
 // g): one batch of record loads, one batch of value loads, then the group sums of all
 // lanes at once, and the group products added in group order by shuffles. With FMA the
-// row is one ordered chain, handed from lane to lane. The operations and their order are
+// row is one ordered chain, handed from lane to lane; in FP64 each lane's turn takes as many
+// operations as the longest of the warp's groups in that place, no more: with turns padded to
+// four or eight, rows of many one-term groups (cubic transfers on an 8 x 8 lattice, 49
+// groups) took 13.6 us a residual and 26.6 a sweep, 8.4 and 17.0 by one thread a node; now 6.0
+// and 11.5 (steps of levels with 45 terms: 0.69 of the padded form). The operations and their order are
 // those of RowSum, so the results are the same bits; a 45-point FP64 row takes about 20
 // warp instructions of FP64 instead of 60, and about 250 instructions in all (a lone warp
 // spends 8-16 clocks on each). A first form that staged records and values in shared
-// memory and summed from there took 600 instructions; see kernels.cu for both timings.
+// memory and summed from there took 600 instructions.
 #pragma once
 
 #include "device.cuh"
@@ -188,15 +192,31 @@ __device__ __forceinline__ T octet_row(const LevelGeo<T>& L, const T* own, const
         for (int t = 0; t < kOct; ++t)
           if (t < ng) s = Arith<T>::add(s, __shfl_sync(0xffffffffu, p, t, kOct));
       } else {
+        // terms of the turns in FP64, four bits each: the most among the warp's octets
+        uint32_t turns = 0;
+        if constexpr (sizeof(T) == 8) {
+          int c = max(r[k].cnt, __shfl_xor_sync(0xffffffffu, r[k].cnt, 8));
+          c = max(c, __shfl_xor_sync(0xffffffffu, c, 16));
+          turns = __reduce_or_sync(0xffffffffu, (uint32_t)c << (4 * l8));
+        }
 #pragma unroll
         for (int t = 0; t < kOct; ++t) {
           if (t >= ng) break;
           T v = s;
+          if constexpr (sizeof(T) == 8) {
+            const int c = (int)(turns >> (4 * t)) & 15;
 #pragma unroll
-          for (int m = 0; m < 4; ++m) v = Arith<T>::fma(r[k].c, x[k][m], v);
-          if (mx > 4) {
+            for (int m = 0; m < kGroupMax; ++m) {
+              if (m >= c) break;
+              v = Arith<T>::fma(r[k].c, x[k][m], v);
+            }
+          } else {
 #pragma unroll
-            for (int m = 4; m < kGroupMax; ++m) v = Arith<T>::fma(r[k].c, x[k][m], v);
+            for (int m = 0; m < 4; ++m) v = Arith<T>::fma(r[k].c, x[k][m], v);
+            if (mx > 4) {
+#pragma unroll
+              for (int m = 4; m < kGroupMax; ++m) v = Arith<T>::fma(r[k].c, x[k][m], v);
+            }
           }
           s = __shfl_sync(0xffffffffu, v, t, kOct);
         }

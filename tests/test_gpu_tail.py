@@ -107,3 +107,23 @@ def test_v_cycles_with_one_kernel_sweeps_have_a_tail(setting, fma, precision):
     u2, hist2, launches2 = solve(setting, "rb2", tail_unknowns=-1, **o)
     assert np.array_equal(u, u2) and hist == hist2
     assert launches < launches2
+
+
+@pytest.mark.parametrize("boundary", ["dirichlet", "periodic"])
+@pytest.mark.parametrize("n", [16, 64])
+def test_fma_rows_of_cubic_transfers_by_octets_and_by_threads(n, boundary):
+    """Rows of up to 121 terms in groups of one to eight: an octet of lanes hands the FMA sum from
+    lane to lane (separate launches), a thread walks it term by term (tail); the same bits."""
+    f = synth.rhs_periodic_normal(n, seed=7) if boundary == "periodic" else synth.rhs_normal(n, seed=7)
+    out = []
+    for tail in (0, -1):
+        u = torch.zeros((n + 1, n + 1), dtype=torch.float64, device="cuda")
+        h = mg.mg_setup(n, 4, STANDARD, GALERKIN, nu1=2, gamma=2, fma_contract=1, transfer_order=4, boundary=boundary,
+                        tail_unknowns=tail)
+        try:
+            _, hist = mg.mg_solve(h, u, torch.tensor(f, device="cuda"), rtol=0.0, max_cycles=CYCLES,
+                                  raise_not_converged=False)
+        finally:
+            h.close()
+        out.append((u.cpu().numpy(), hist))
+    assert np.array_equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
