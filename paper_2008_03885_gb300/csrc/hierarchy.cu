@@ -1996,7 +1996,6 @@ mg_status build_lists(mg_batch* b, std::vector<BatchList<T>>& lv) {
       e.coarsest_idx = H.coarsest_idx;
       e.coarsest_a = H.coarsest_a;
       e.dense = H.dense;
-      e.dc = H.d[l + 1];
       B.host.push_back(e);
       if (l + 2 == nlp) (H.dense.m > 0 ? coarsest_dense : coarsest).push_back(e);
     }

@@ -1996,7 +1996,6 @@ cudaError_t launch_half_sweep(const LevelPair<T>& L, bool exact, const T* uin, c
     if (exact) return launch_pdl<T>(k_half_sweep_gen<T, true, false>, g, b, s, A, uin, f, uout);
     else return launch_pdl<T>(k_half_sweep_gen<T, false, false>, g, b, s, A, uin, f, uout);
   }
-  return cudaGetLastError();
 }
 
 template <typename T, bool EXACT, int NT>
@@ -2082,7 +2081,6 @@ cudaError_t launch_residual(const LevelPair<T>& L, bool exact, const T* u, const
     if (exact) return launch_pdl<T>(k_residual_gen<T, true, false>, g, b, s, A, u, f, d);
     else return launch_pdl<T>(k_residual_gen<T, false, false>, g, b, s, A, u, f, d);
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -2118,7 +2116,6 @@ cudaError_t launch_restrict(const LevelPair<T>& Lf, const LevelPair<T>& Lc, int 
     if (exact) return launch_pdl<T>(k_restrict<T, true, false, 1>, g, b, s, Lf.h, Lc.h, transfer, d, fc, tc);
     else return launch_pdl<T>(k_restrict<T, false, false, 1>, g, b, s, Lf.h, Lc.h, transfer, d, fc, tc);
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -2155,7 +2152,6 @@ cudaError_t launch_prolong_add(const LevelPair<T>& Lf, const LevelPair<T>& Lc, i
     if (exact) return launch_pdl<T>(k_prolong_add<T, true, false, 1, false>, g, b, s, Lf.h, Lc.h, transfer, ui, uf, vc);
     else return launch_pdl<T>(k_prolong_add<T, false, false, 1, false>, g, b, s, Lf.h, Lc.h, transfer, ui, uf, vc);
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -2164,7 +2160,6 @@ cudaError_t launch_coarsest_dense(const DenseCoarse<T>& C, const LevelPair<T>& L
   const int threads = std::min(1024, (C.m + 31) / 32 * 32);
   if (exact) return launch_pdl<T>(k_coarsest_dense<T, true>, 1, threads, s, C, L.h, f, u);
   else return launch_pdl<T>(k_coarsest_dense<T, false>, 1, threads, s, C, L.h, f, u);
-  return cudaGetLastError();
 }
 
 template <typename T>

@@ -164,8 +164,7 @@ struct BatchLevel {
   int32_t tiles_x, ctiles_x;  // tiles per row of tiles on level l / level l + 1
   int64_t coarsest_idx;   // of level l + 1 when it is the problem's coarsest level
   T coarsest_a;
-  DenseCoarse<T> dense;   //   m > 0: its dense solve (y in dc)
-  T* dc;                  // level l + 1's d array
+  DenseCoarse<T> dense;   //   m > 0: its dense solve
   float* r32;             // finest level, mixed precision: FP32 residual (inner right-hand side)
   float* e32;             //   and FP32 correction
   int32_t pitch32;        //   row pitch of those FP32 arrays (padded to 32 elements)
