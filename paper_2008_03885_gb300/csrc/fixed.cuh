@@ -83,7 +83,7 @@ __device__ __forceinline__ float scaled_float(double r, int k, double scale) {
 
 struct FxSmem {
   int64_t q[2][kFxRegion];  // u, then its fixed-point values, of this tile and the next
-  uint32_t red[3][8];
+  uint32_t red[2][8];
 };
 
 // Copies u of the region of tile (i0, j0) to `dst` asynchronously, boundary values (unless
@@ -128,40 +128,35 @@ __device__ __forceinline__ void fx_tile(const LevelGeo<double>& L, const LevelDe
     const int j = j0 + r0 + r;
     fv[r] = i >= 1 && i < n && j < n ? f[(int64_t)j * L.pitch + i] : 0.0;
   }
-  // largest high word, smallest one less 1 (zeros, and values below 2^-1042, which reach neither
-  // the FP32 residual nor the norm, wrap to the largest), any bit
-  uint32_t mx = 0, mn = ~0u, any = 0;
+  // largest high word, and the smallest one less 1 (zeros wrap to the largest); values below
+  // 2^-1042 count as 0: they reach neither the FP32 residual nor the norm
+  uint32_t mx = 0, mn = ~0u;
 #pragma unroll
   for (int k = 0; k < kFxPer; ++k) {
     if (tid + 256 * k >= kFxRegion) break;
-    const uint64_t v = (uint64_t)buf[tid + 256 * k];
-    const uint32_t h = (uint32_t)(v >> 32) & 0x7fffffffu;
+    const uint32_t h = (uint32_t)((uint64_t)buf[tid + 256 * k] >> 32) & 0x7fffffffu;
     mx = max(mx, h);
     mn = min(mn, h - 1);
-    any |= h | (uint32_t)v;
   }
   mx = __reduce_max_sync(0xffffffffu, mx);
   mn = __reduce_min_sync(0xffffffffu, mn);
-  any = __reduce_or_sync(0xffffffffu, any);
   if (threadIdx.x == 0) {
     sm.red[0][threadIdx.y] = mx;
-    sm.red[1][threadIdx.y] = any;
-    sm.red[2][threadIdx.y] = mn;
+    sm.red[1][threadIdx.y] = mn;
   }
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     mx = max(mx, sm.red[0][k]);
-    any |= sm.red[1][k];
-    mn = min(mn, sm.red[2][k]);
+    mn = min(mn, sm.red[1][k]);
   }
   const int E = (int)(mx >> 20);
   uint32_t rest = 0;  // bit r: the node of row r takes its FP64 row
-  if (any != 0 && (E == 0x7ff || E < 128)) {  // uniform over the block
+  if (mx != 0 && (E == 0x7ff || E < 128)) {  // uniform over the block
     rest = (1u << kRows) - 1;
   } else {
     // whether some value may lose bits (uniform over the block)
-    const bool marks = (int)((mx >> 20) - ((mn + 1) >> 20)) > kFxS0 && mn != ~0u;
+    const bool marks = mx != 0 && E - (int)((mn + 1) >> 20) > kFxS0;
     auto convert = [&](auto mark) {
 #pragma unroll
       for (int k = 0; k < kFxPer; ++k) {
@@ -169,17 +164,17 @@ __device__ __forceinline__ void fx_tile(const LevelGeo<double>& L, const LevelDe
         buf[tid + 256 * k] = to_fixed<decltype(mark)::value>(__longlong_as_double(buf[tid + 256 * k]), E);
       }
     };
-    if (any != 0) {
+    if (mx != 0) {
       if (marks) convert(std::true_type());
       else convert(std::false_type());
     }
     __syncthreads();
-    // L u = c0 T, T in units of 2^(E - 1075 - kFxS0 - 1) (any != 0: E >= 128, so the factor is
-    // normal; any == 0: the region holds zeros)
-    const double unit = any != 0 ? -L.c0 * __hiloint2double((E - 53 - kFxS0) << 20, 0) : 0.0;
-    // Most tiles need no marks and run without the tests: 8193^2, order 2, solved u: 554 us
+    // L u = c0 T, T in units of 2^(E - 1075 - kFxS0 - 1) (mx != 0: E >= 128, so the factor is
+    // normal; mx == 0: the region holds zeros)
+    const double unit = mx != 0 ? -L.c0 * __hiloint2double((E - 53 - kFxS0) << 20, 0) : 0.0;
+    // Most tiles need no marks and run without the tests: 8193^2, order 2, solved u: 545 us
     // (595 with marks in every tile, 515 with none at all, bits lost; white noise, where most
-    // warps hold a marked row, 1005; FP64 rows 1208)
+    // warps hold a marked row, 995; FP64 rows 1208)
     auto walk = [&](auto marked) {
       const int64_t* q = buf + (r0 + 1) * W + cx + 1;
       int64_t below = q[-W], here = q[0];

@@ -1244,7 +1244,7 @@ __global__ void __launch_bounds__(kBX * kBY, MinBlocks<double>::value)
 // The refinement residual in fixed point (fixed.cuh), the tiles in a flat order over one
 // resident wave as k_ir_residual's, the next tile's u in flight during the current one's
 // work (without: 709 us at 8193^2, order 2, with 3 blocks per SM; 502 with 4, both before
-// values were tested for lost bits: 554 now). FP64 rows took 1208 us there; 200 us of HBM are
+// values were tested for lost bits: 545 now). FP64 rows took 1208 us there; 200 us of HBM are
 // its floor, integer issue and the waits between its phases what bounds it.
 template <bool EXACT>
 __global__ void __launch_bounds__(kBX * kBY, 4)
